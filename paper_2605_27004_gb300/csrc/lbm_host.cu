@@ -18,10 +18,10 @@
 
 namespace lbm {
 
-Shape shape_for(const Geom& g, int nzp) {
+Shape shape_for(const Geom& g, int nzp, int threads) {
     Shape s;
-    const int bx = block_x_for(g.nx);
-    const int by = std::max(1, 256 / bx);
+    const int bx = block_x_for(g.nx, threads);
+    const int by = std::max(1, threads / bx);
     s.block = dim3(bx, by, 1);
     s.grid = dim3((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, nzp);
     s.nblocks = (long long)s.grid.x * s.grid.y * s.grid.z;

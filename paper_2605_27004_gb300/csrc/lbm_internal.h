@@ -63,7 +63,7 @@ struct Shape {
     dim3 grid, block;
     long long nblocks;
 };
-Shape shape_for(const Geom& g, int nzp);
+Shape shape_for(const Geom& g, int nzp, int threads = 256);
 
 // Block width for n threads along x: a multiple of 32 up to 256 that wastes the fewest threads
 // in the last block of a row; among those, a divisor of 256 (so that blocks of bx x 256/bx

@@ -182,8 +182,8 @@ __device__ __forceinline__ uint32_t link_of(const Geom& g, const Cell& c) {
 }
 __device__ __forceinline__ bool link_bit(uint32_t lw, int i) { return (lw >> i) & 1u; }
 
-// Gather of the pre-collision populations of one cell in shifted form (see Layout).
-template <int Q, int S, bool MASK, int LAYOUT, bool RO>
+// Gather of the pre-collision populations of one cell in shifted form (see Layout); RAW: as stored.
+template <int Q, int S, bool MASK, int LAYOUT, bool RO, bool RAW = false>
 __device__ __forceinline__ void gather(const Cell& c, uint32_t lw, const Coef<typename Store<S>::T>& cf,
                                        const Planes<const typename Store<S>::type>& src,
                                        typename Store<S>::T (&d)[Q]) {
@@ -210,7 +210,7 @@ __device__ __forceinline__ void gather(const Cell& c, uint32_t lw, const Coef<ty
             }
         }
         const auto raw = RO ? ld_ro(p) : ld_rw(p);
-        d[i] = to_shifted<S>(raw, cf.so[i]);
+        d[i] = RAW ? raw : to_shifted<S>(raw, cf.so[i]);
     }
 }
 
@@ -365,6 +365,107 @@ __device__ __forceinline__ Macro<T> bgk(const Coef<T>& cf, T (&d)[Q]) {
     return m;
 }
 
+// ---------------------------------------------------------------------------------------------
+// BGK collision of FP64 storage, in place on the stored populations f_i. The FP64 kernels are bound
+// by the FP64 pipe (two fused multiply-adds per SM and clock: 85 % busy at 64^3 with the shifted
+// form above, 263 FP64 instructions per D3Q19 cell, while DRAM is 4 % busy), so this form counts
+// operations: no shift on load and store (FP64 keeps f ~ w_i to 1e-16; om rho A_i is om feq's
+// density part and r_i at once), 1/tau folded into per-cell factors, and (c.u)^2 of axes and edges
+// from shared products (edge: u_a^2 + u_b^2 +- 2 u_a u_b; minus |u|^2 it is +- 2 u_a u_b - u_c^2).
+// About 200 a cell: D3Q19 64^3 137 -> 98.6 us a step.
+// ---------------------------------------------------------------------------------------------
+template <int Q>
+__device__ __forceinline__ Macro<double> bgk_raw(const Coef<double>& cf, double (&f)[Q]) {
+    constexpr bool D3 = Lat<Q>::D == 3;
+    double s = f[0], j[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < Lat<Q>::P; ++k) {
+        const Vec3 v = vel<Q>(2 * k + 1);
+        const double a = f[2 * k + 1], b = f[2 * k + 2], o = a - b;
+        const int n = v.x * v.x + v.y * v.y + v.z * v.z;
+        s += a + b;
+        // the axis pairs come first and start the sums
+        if (v.x) j[0] = n == 1 ? o : (v.x > 0 ? j[0] + o : j[0] - o);
+        if (v.y) j[1] = n == 1 ? o : (v.y > 0 ? j[1] + o : j[1] - o);
+        if (v.z) j[2] = n == 1 ? o : (v.z > 0 ? j[2] + o : j[2] - o);
+    }
+    Macro<double> m;
+    m.rho = s;
+    m.drho = 0.0;  // not used in this form
+    m.jx = j[0];
+    m.jy = j[1];
+    m.jz = j[2];
+    const double inv = 1.0 / s;
+    m.ux = j[0] * inv;
+    m.uy = j[1] * inv;
+    m.uz = D3 ? j[2] * inv : 0.0;
+    const double om1 = 1.0 - cf.omega, omrho = cf.omega * s;
+    const double u[3] = {m.ux, m.uy, m.uz};
+    const double q[3] = {u[0] * u[0], u[1] * u[1], D3 ? u[2] * u[2] : 0.0};
+    const double sum[3] = {D3 ? q[1] + q[2] : q[1], D3 ? q[0] + q[2] : q[0], q[0] + q[1]};  // |u|^2 - u_a^2
+    const double usq = D3 ? sum[2] + q[2] : sum[2];
+    const double x2 = u[0] + u[0], y2 = u[1] + u[1];
+    const double prod[3] = {D3 ? y2 * u[2] : 0.0, D3 ? x2 * u[2] : 0.0, x2 * u[1]};  // 2 u_b u_c, a the third axis
+    const double kz = D3 ? fma(cf.K[4], u[0], fma(cf.K[5], u[1], cf.K[2] * u[2])) : 0.0;
+    const double kx = fma(cf.K[0], u[0], D3 ? fma(cf.K[3], u[1], cf.K[4] * u[2]) : cf.K[3] * u[1]);
+    const double ky = fma(cf.K[3], u[0], D3 ? fma(cf.K[1], u[1], cf.K[5] * u[2]) : cf.K[1] * u[1]);
+    const double r45 = 4.5 * omrho, r15 = r45 * usq * (1.0 / 3.0), rc3 = cf.c3 * omrho;
+    f[0] = fma(om1, f[0], fma(omrho, cf.A[0], -(weight<Q>(0) * r15)));
+#pragma unroll
+    for (int k = 0; k < Lat<Q>::P; ++k) {
+        const int i = 2 * k + 1;
+        const Vec3 v = vel<Q>(i);
+        const int n = v.x * v.x + v.y * v.y + v.z * v.z;
+        const double w = weight<Q>(i);
+        const double a = w * r45, base = w * r15, b = w * rc3;  // one value per |c|^2
+        const double bx = (b + b) * kx, by = (b + b) * ky, bz = D3 ? (b + b) * kz : 0.0;
+        double uc, uc2, g, bk;  // c.u, (c.u)^2, (c.u)^2 - |u|^2, 2 b c.K~u
+        if (n == 1) {
+            const int e = v.x ? 0 : v.y ? 1 : 2;
+            uc = u[e];
+            uc2 = q[e];
+            g = -sum[e];
+            bk = v.x ? bx : v.y ? by : bz;
+        } else if (n == 2) {
+            // half-vectors have +1 first: (+a, +b) or (+a, -b)
+            const int e = v.x == 0 ? 0 : v.y == 0 ? 1 : 2;
+            const double first = v.x ? u[0] : u[1], second = v.z ? u[2] : u[1];
+            const double bf = v.x ? bx : by, bs = v.z ? bz : by;
+            const bool plus = (v.x ? v.x : v.y) * (v.z ? v.z : v.y) > 0;
+            uc = plus ? first + second : first - second;
+            uc2 = plus ? sum[e] + prod[e] : sum[e] - prod[e];
+            g = Lat<Q>::D == 3 ? (plus ? prod[e] - q[e] : -prod[e] - q[e]) : (plus ? prod[e] : -prod[e]);
+            bk = plus ? bf + bs : bf - bs;
+        } else {
+            const double uxy = v.y > 0 ? u[0] + u[1] : u[0] - u[1], bxy = v.y > 0 ? bx + by : bx - by;
+            uc = v.z > 0 ? uxy + u[2] : uxy - u[2];
+            uc2 = uc * uc;
+            g = uc2 - usq;
+            bk = v.z > 0 ? bxy + bz : bxy - bz;
+        }
+        const double E = fma(a, uc2, fma(omrho, cf.A[i], -base));
+        const double O = fma(uc, fma(b, g, omrho * cf.B[i]), -bk);
+        f[i] = fma(om1, f[i], E + O);
+        f[i + 1] = fma(om1, f[i + 1], E - O);
+    }
+    return m;
+}
+
+// The collision of a flow step on gathered populations: FP64 storage as stored, the others shifted.
+template <int Q, int S>
+__device__ __forceinline__ Macro<typename Store<S>::T> collide(const Coef<typename Store<S>::T>& cf,
+                                                               typename Store<S>::T (&d)[Q]) {
+    if constexpr (S == 1)
+        return bgk_raw<Q>(cf, d);
+    else
+        return bgk<Q, typename Store<S>::T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+}
+// the stored value of a collided population
+template <int S>
+__device__ __forceinline__ typename Store<S>::T stored(typename Store<S>::T d, typename Store<S>::T so) {
+    return S == 1 ? d : from_shifted<S>(d, so);
+}
+
 template <typename T>
 __device__ __forceinline__ bool bad_cell(const Macro<T>& m) {
     return !(m.rho > T(0)) || !isfinite(m.ux + m.uy + m.uz);
@@ -406,18 +507,18 @@ __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S
     if (MASK && __all_sync(act, lw == 0u)) {
         // no lane of the warp has a wall link: the branch-free gather (in the porous medium of
         // overlapping spheres about 28 % of the warps, 40 % of the fluid cells)
-        gather<Q, S, false, LAYOUT_PULL, true>(c, 0u, cf, src, d);
+        gather<Q, S, false, LAYOUT_PULL, true, S == 1>(c, 0u, cf, src, d);
     } else if (!solid) {
-        gather<Q, S, MASK, LAYOUT_PULL, true>(c, lw, cf, src, d);
+        gather<Q, S, MASK, LAYOUT_PULL, true, S == 1>(c, lw, cf, src, d);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
     }
-    const Macro<T> m = bgk<Q, T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+    const Macro<T> m = collide<Q, S>(cf, d);
     if (!solid && bad_cell(m)) *flag = 1;
     if (MASK && !store_group<typename Store<S>::type>(act, solid)) return;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : from_shifted<S>(d[i], cf.so[i]));
+    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : stored<S>(d[i], cf.so[i]));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -446,7 +547,7 @@ __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<
             else
                 p = dst.p[i] + off_plus(c, v);
         }
-        st_raw(p, from_shifted<S>(d[i], cf.so[i]));
+        st_raw(p, stored<S>(d[i], cf.so[i]));
     }
 }
 
@@ -464,15 +565,15 @@ __global__ void __launch_bounds__(256) k_step_aa(Geom g, Coef<typename Store<S>:
     const bool clean = MASK && __all_sync(__activemask(), lw == 0u);
     if (clean) {
         if (ODD)
-            gather<Q, S, false, LAYOUT_AAODD, false>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_AAODD, false, S == 1>(c, 0u, cf, src, d);
         else
-            gather<Q, S, false, LAYOUT_LOCAL, false>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_LOCAL, false, S == 1>(c, 0u, cf, src, d);
     } else if (ODD) {
-        gather<Q, S, MASK, LAYOUT_AAODD, false>(c, lw, cf, src, d);
+        gather<Q, S, MASK, LAYOUT_AAODD, false, S == 1>(c, lw, cf, src, d);
     } else {
-        gather<Q, S, MASK, LAYOUT_LOCAL, false>(c, lw, cf, src, d);
+        gather<Q, S, MASK, LAYOUT_LOCAL, false, S == 1>(c, lw, cf, src, d);
     }
-    const Macro<T> m = bgk<Q, T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+    const Macro<T> m = collide<Q, S>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
         aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);
@@ -548,19 +649,19 @@ __global__ void __launch_bounds__(256) k_step_pull_sectors(Geom g, Coef<typename
     if (__all_sync(act, solid)) return;
     T d[Q];
     if (__all_sync(act, lw == 0u)) {
-        gather<Q, S, false, LAYOUT_PULL, true>(c, 0u, cf, src, d);
+        gather<Q, S, false, LAYOUT_PULL, true, S == 1>(c, 0u, cf, src, d);
     } else if (!solid) {
-        gather<Q, S, true, LAYOUT_PULL, true>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_PULL, true, S == 1>(c, lw, cf, src, d);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
     }
-    const Macro<T> m = bgk<Q, T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+    const Macro<T> m = collide<Q, S>(cf, d);
     if (!solid && bad_cell(m)) *flag = 1;
     const bool store = store_group<typename Store<S>::type>(act, solid);
     if (!valid || !store) return;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : from_shifted<S>(d[i], cf.so[i]));
+    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : stored<S>(d[i], cf.so[i]));
 }
 
 template <int Q, int S, int ODD>
@@ -576,15 +677,15 @@ __global__ void __launch_bounds__(256, 4) k_step_aa_list(Geom g, Coef<typename S
     const bool clean = __all_sync(__activemask(), lw == 0u);
     if (clean) {
         if (ODD)
-            gather<Q, S, false, LAYOUT_AAODD, false>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_AAODD, false, S == 1>(c, 0u, cf, src, d);
         else
-            gather<Q, S, false, LAYOUT_LOCAL, false>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_LOCAL, false, S == 1>(c, 0u, cf, src, d);
     } else if (ODD) {
-        gather<Q, S, true, LAYOUT_AAODD, false>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_AAODD, false, S == 1>(c, lw, cf, src, d);
     } else {
-        gather<Q, S, true, LAYOUT_LOCAL, false>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_LOCAL, false, S == 1>(c, lw, cf, src, d);
     }
-    const Macro<T> m = bgk<Q, T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+    const Macro<T> m = collide<Q, S>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
         aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);

@@ -56,9 +56,22 @@ struct Launch {
     // populations per thread and stays at two cells.
     static bool quads(const Geom& g) { return S == 3 && Q != 27 && !g.link && (g.nx % 128) == 0; }
 
+    // FP64 steps are bound by the FP64 pipes, so their blocks have 64 threads: a small box then
+    // reaches every SM (64^2 ran on 16 of them: 11.2 -> 4.6 us a step with the FP64 collision of
+    // bgk_raw; 33 x 29 x 41 37.3 -> 29.5 us against 256 threads; from 64^3 up there is no
+    // difference). A box too tall for 64-thread blocks (grid.y) keeps 256.
+    static Shape shape_step(const Geom& g) {
+        const int nzp = g.nz - 2 * LBM_SLAB;
+        if (S == 1) {
+            const Shape small = shape_for(g, nzp, 64);
+            if (small.grid.y <= 65535u) return small;
+        }
+        return shape_for(g, nzp);
+    }
+
     static cudaError_t step_pull(const Geom& g, const void* coef, const void* src, void* dst, int* flag,
                                  cudaStream_t st) {
-        const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
+        const Shape sh = shape_step(g);
         const CF& cf = *static_cast<const CF*>(coef);
         const auto a = cpl(src, g);
         const auto b = mpl(dst, g);
@@ -85,7 +98,7 @@ struct Launch {
 
     static cudaError_t step_aa(const Geom& g, const void* coef, int odd, const void* src, void* dst, int* flag,
                                cudaStream_t st) {
-        const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
+        const Shape sh = shape_step(g);
         const CF& cf = *static_cast<const CF*>(coef);
         const auto a = cpl(src, g);
         const auto b = mpl(dst, g);
