@@ -26,13 +26,13 @@ struct VelField {
 };
 
 // Relaxes d in place towards geq(phi, u(x)); returns phi - rho0 (phi0 of the shifted storage).
-template <int Q, typename T>
+template <int Q, bool EARLY, typename T>
 __device__ __forceinline__ T ade_bgk(const Coef<T>& cf, const VelField<T>& vf, uint32_t n, T (&d)[Q]) {
     T ux = T(0), uy = T(0), uz = T(0);
     if (vf.p[0] != nullptr) {
-        ux = ld_ro(vf.p[0] + n);
-        uy = ld_ro(vf.p[1] + n);
-        if (Lat<Q>::D == 3) uz = ld_ro(vf.p[2] + n);
+        ux = EARLY ? ld_rw(vf.p[0] + n) : ld_ro(vf.p[0] + n);
+        uy = EARLY ? ld_rw(vf.p[1] + n) : ld_ro(vf.p[1] + n);
+        if (Lat<Q>::D == 3) uz = EARLY ? ld_rw(vf.p[2] + n) : ld_ro(vf.p[2] + n);
     }
     T s = d[0];
 #pragma unroll
@@ -43,7 +43,7 @@ __device__ __forceinline__ T ade_bgk(const Coef<T>& cf, const VelField<T>& vf, u
 }
 
 // Fused stream + collide of the scalar populations, two arrays, pull form (see k_step_pull).
-template <int Q, int S, bool MASK>
+template <int Q, int S, bool MASK, bool EARLY>
 __global__ void __launch_bounds__(256)
     k_ade_pull(Geom g, Coef<typename Store<S>::T> cf, VelField<typename Store<S>::T> vf,
                const Planes<const typename Store<S>::type> src, const Planes<typename Store<S>::type> dst,
@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256)
     using T = typename Store<S>::T;
     Cell c;
     if (!make_cell(g, c)) return;
+    wait_previous<EARLY>();
     const uint32_t lw = link_of<MASK>(g, c);
     // with walls, solid lanes of a sector that holds a fluid cell store zeros into their own
     // (never read) slots, so that destination sectors are written whole (as in k_step_pull)
@@ -59,14 +60,14 @@ __global__ void __launch_bounds__(256)
     if (MASK && __all_sync(act, solid)) return;
     T d[Q];
     if (MASK && __all_sync(act, lw == 0u)) {  // no wall link in the warp (see k_step_pull)
-        gather<Q, S, false, LAYOUT_PULL, true>(c, 0u, cf, src, d);
+        gather<Q, S, false, LAYOUT_PULL, !EARLY>(c, 0u, cf, src, d);
     } else if (!solid) {
-        gather<Q, S, MASK, LAYOUT_PULL, true>(c, lw, cf, src, d);
+        gather<Q, S, MASK, LAYOUT_PULL, !EARLY>(c, lw, cf, src, d);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
     }
-    const T s = ade_bgk<Q, T>(cf, vf, c.n, d);
+    const T s = ade_bgk<Q, EARLY>(cf, vf, c.n, d);
     if (!solid && !isfinite(s)) *flag = 1;
     if (MASK && !store_group<typename Store<S>::type>(act, solid)) return;
 #pragma unroll
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
     }
-    const T s = ade_bgk<Q, T>(cf, vf, c.n, d);
+    const T s = ade_bgk<Q, false>(cf, vf, c.n, d);
     if (!solid && !isfinite(s)) *flag = 1;
     const bool store = store_group<typename Store<S>::type>(act, solid);
     if (!valid || !store) return;
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(256)
 
 // AA pattern in place (see k_step_aa): even steps read and write the own cell, odd steps the
 // neighbours along +c_i.
-template <int Q, int S, bool MASK, int ODD>
+template <int Q, int S, bool MASK, int ODD, bool EARLY>
 __global__ void __launch_bounds__(256)
     k_ade_aa(Geom g, Coef<typename Store<S>::T> cf, VelField<typename Store<S>::T> vf,
              const Planes<const typename Store<S>::type> src, const Planes<typename Store<S>::type> dst,
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(256)
     using T = typename Store<S>::T;
     Cell c;
     if (!make_cell(g, c)) return;
+    wait_previous<EARLY>();
     const uint32_t lw = link_of<MASK>(g, c);
     if (MASK && (lw & LINK_SOLID)) return;
     T d[Q];
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(256)
     } else {
         gather<Q, S, MASK, LAYOUT_LOCAL, false>(c, lw, cf, src, d);
     }
-    const T s = ade_bgk<Q, T>(cf, vf, c.n, d);
+    const T s = ade_bgk<Q, EARLY>(cf, vf, c.n, d);
     if (!isfinite(s)) *flag = 1;
     if (clean)
         aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);

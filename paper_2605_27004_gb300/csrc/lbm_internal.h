@@ -85,6 +85,24 @@ inline int block_x_for(int n, int threads = 256) {
     return best;
 }
 
+// Launch of a kernel that waits for the previous one itself (wait_previous) before its first access
+// to memory that another kernel writes: its blocks may be set up while that one drains.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
 // Kernel launchers of one (lattice, storage) pair. `coef` points at a Coef<double> (storage
 // LBM_FP64) or a Coef<float> (every other storage). Field pointers (rho, u, Pi, f, grad, lam,
 // du0) are double for FP64 and float otherwise; population pointers have the storage type.

@@ -125,6 +125,23 @@ __device__ __forceinline__ typename Store<S>::T from_shifted(typename Store<S>::
     return Store<S>::shifted ? d : d + r;
 }
 
+// The EARLY instances of the per-cell kernels (small boxes: early() in lbm_launch.cuh) are launched
+// with launch_after() and call this once their cell is addressed: it lets the next kernel's blocks be
+// set up as soon as all of this one's have started, and waits for the previous kernel's writes. They
+// read populations, lambda and velocities with ordinary loads, since a non-coherent load may be moved
+// above the wait, and pointers whose memory another kernel writes are not declared __restrict__.
+// Measured per step: D2Q9 64^2 1.67 -> 1.54 us, D3Q19 64^3 FP32 6.3 -> 5.6 us (graph launches), three
+// launches of a flow coupled to a scalar at 96 x 88 x 80 53 -> 44 us. Above 2M cells the wait at the
+// head of every block costs more than the overlap gives (D3Q27 FP32 256^3 521 -> 542 us, D3Q19 FP16
+// 320^3 441 -> 487 us), so larger boxes keep the plain instances.
+template <bool EARLY>
+__device__ __forceinline__ void wait_previous() {
+    if constexpr (EARLY) {
+        cudaTriggerProgrammaticLaunchCompletion();
+        cudaGridDependencySynchronize();
+    }
+}
+
 // Base pointers of the q planes of a structure-of-arrays buffer, passed by value as a kernel
 // parameter so that the bases stay in the constant bank instead of occupying registers.
 template <typename P>
@@ -489,13 +506,14 @@ __device__ __forceinline__ bool store_group(unsigned act, bool solid) {
 // Fused stream + collide, two arrays, pull form: gather f(t) from the post-collision array of
 // the previous step, relax, store at the own cell. One launch per time step.
 // ---------------------------------------------------------------------------------------------
-template <int Q, int S, bool MASK>
+template <int Q, int S, bool MASK, bool EARLY>
 __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S>::T> cf,
                                                    const Planes<const typename Store<S>::type> src,
                                                    const Planes<typename Store<S>::type> dst, int* __restrict__ flag) {
     using T = typename Store<S>::T;
     Cell c;
     if (!make_cell(g, c)) return;
+    wait_previous<EARLY>();
     const uint32_t lw = link_of<MASK>(g, c);
     // With walls, a solid cell's slots are never read (a gather that meets a solid neighbour takes
     // the own cell's opposite slot) nor written by another cell, so a solid lane may store zeros
@@ -507,9 +525,9 @@ __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S
     if (MASK && __all_sync(act, lw == 0u)) {
         // no lane of the warp has a wall link: the branch-free gather (in the porous medium of
         // overlapping spheres about 28 % of the warps, 40 % of the fluid cells)
-        gather<Q, S, false, LAYOUT_PULL, true, S == 1>(c, 0u, cf, src, d);
+        gather<Q, S, false, LAYOUT_PULL, !EARLY, S == 1>(c, 0u, cf, src, d);
     } else if (!solid) {
-        gather<Q, S, MASK, LAYOUT_PULL, true, S == 1>(c, lw, cf, src, d);
+        gather<Q, S, MASK, LAYOUT_PULL, !EARLY, S == 1>(c, lw, cf, src, d);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
@@ -551,13 +569,14 @@ __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<
     }
 }
 
-template <int Q, int S, bool MASK, int ODD>
+template <int Q, int S, bool MASK, int ODD, bool EARLY>
 __global__ void __launch_bounds__(256) k_step_aa(Geom g, Coef<typename Store<S>::T> cf,
                                                  const Planes<const typename Store<S>::type> src,
                                                  const Planes<typename Store<S>::type> dst, int* __restrict__ flag) {
     using T = typename Store<S>::T;
     Cell c;
     if (!make_cell(g, c)) return;
+    wait_previous<EARLY>();
     const uint32_t lw = link_of<MASK>(g, c);
     if (MASK && (lw & LINK_SOLID)) return;
     T d[Q];
@@ -766,18 +785,19 @@ __host__ __device__ constexpr int pi_b(int D, int k) {
 __host__ __device__ constexpr int pi_full(int D, int k) { return D == 2 ? (k == 2 ? 3 : k) : k; }
 __host__ __device__ constexpr int comp(Vec3 v, int a) { return a == 0 ? v.x : a == 1 ? v.y : v.z; }
 
-template <int Q, int S, bool MASK, int LAYOUT>
+template <int Q, int S, bool MASK, int LAYOUT, bool EARLY>
 __global__ void __launch_bounds__(256) k_moments(Geom g, Coef<typename Store<S>::T> cf,
                                                  const Planes<const typename Store<S>::type> src,
-                                                 typename Store<S>::T* __restrict__ rho_out,
-                                                 typename Store<S>::T* __restrict__ u_out,
-                                                 typename Store<S>::T* __restrict__ pi_out,
-                                                 typename Store<S>::T* __restrict__ f_out) {
+                                                 typename Store<S>::T* rho_out,
+                                                 typename Store<S>::T* u_out,
+                                                 typename Store<S>::T* pi_out,
+                                                 typename Store<S>::T* f_out) {
     using T = typename Store<S>::T;
     constexpr int D = Lat<Q>::D;
     constexpr int NP = D == 2 ? 3 : 6;
     Cell c;
     if (!make_cell(g, c)) return;
+    wait_previous<EARLY>();
     const size_t N = g.N;
     const uint32_t lw = link_of<MASK>(g, c);
     if (MASK && (lw & LINK_SOLID)) {
@@ -791,7 +811,7 @@ __global__ void __launch_bounds__(256) k_moments(Geom g, Coef<typename Store<S>:
         return;
     }
     T d[Q];
-    gather<Q, S, MASK, LAYOUT, true>(c, lw, cf, src, d);
+    gather<Q, S, MASK, LAYOUT, !EARLY>(c, lw, cf, src, d);
     const Macro<T> m = macro_of<Q, T>(d, cf.rho0);
     if (rho_out) rho_out[c.n] = m.rho;
     if (u_out) {
@@ -1079,15 +1099,16 @@ __global__ void __launch_bounds__(256) k_adj_seed(Geom g, Coef<typename Store<S>
 // spilled values stay in L1): FP16 AA adjoint at 256^3 0.69 -> 0.77 of the copy peak, FP32 pull
 // 0.87 -> 0.90 (measured). D3Q27 at most 128 (two blocks instead of one at 189 registers, no
 // spills). FP64 storage is left uncapped.
-template <int Q, int S, bool MASK, int LAYOUT>
+template <int Q, int S, bool MASK, int LAYOUT, bool EARLY>
 __global__ void __launch_bounds__(256, S == 1 ? 1 : Q == 27 ? 2 : 4) k_adj_step(Geom g, Coef<typename Store<S>::T> cf,
                                                   const Planes<const typename Store<S>::type> src,
                                                   const Planes<const typename Store<S>::T> lam_next,
-                                                  const Planes<typename Store<S>::T> lam, double* __restrict__ gpart) {
+                                                  const Planes<typename Store<S>::T> lam, double* gpart) {
     using T = typename Store<S>::T;
     T rec[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
     Cell c;
     if (make_cell(g, c)) {
+        wait_previous<EARLY>();
         const uint32_t lw = link_of<MASK>(g, c);
         if (!(MASK && (lw & LINK_SOLID))) {
             // mu = S^T lambda_{t+1}: reverse gather along +c_i
@@ -1101,11 +1122,11 @@ __global__ void __launch_bounds__(256, S == 1 ? 1 : Q == 27 ? 2 : 4) k_adj_step(
                     p = lam_next.p[opp(i)] + c.n;
                 else
                     p = lam_next.p[i] + off_plus(c, vel<Q>(i));
-                mu[i] = __ldg(p);
+                mu[i] = EARLY ? *p : __ldg(p);
             }
             // f_t: moments, and f_i itself for the tau-gradient
             T dk[Q];
-            gather<Q, S, MASK, LAYOUT, true>(c, lw, cf, src, dk);
+            gather<Q, S, MASK, LAYOUT, !EARLY>(c, lw, cf, src, dk);
             const Macro<T> m = macro_of<Q, T>(dk, cf.rho0);
             const EqCell<T> e = eq_cell<T>(cf, m.drho, m.rho, m.ux, m.uy, m.uz);
             const AdjAcc<T> A = adj_accumulate<Q, T>(cf, e, mu, dk);

@@ -21,6 +21,15 @@ struct Launch {
     static Planes<const T> cfl(const void* p, const Geom& g) { return planes_of(static_cast<const T*>(p), Q, g.N); }
     static Planes<T> mfl(void* p, const Geom& g) { return planes_of(static_cast<T*>(p), Q, g.N); }
 
+    // Boxes whose kernels take the EARLY instances (wait_previous): the launch gap counts there.
+    static bool early(const Geom& g) { return g.N <= (1u << 21); }
+#define LBM_UNWRAP(...) __VA_ARGS__
+#define LBM_EARLY(K, PARAMS, GRID, BLOCK, ...)                                                     \
+    do {                                                                                           \
+        if (early(g)) return launch_after(K<LBM_UNWRAP PARAMS, true>, GRID, BLOCK, st, __VA_ARGS__); \
+        K<LBM_UNWRAP PARAMS, false><<<GRID, BLOCK, 0, st>>>(__VA_ARGS__);                          \
+    } while (0)
+
     static cudaError_t init(const Geom& g, const void* coef, int layout, const void* rho, const void* u, void* dst,
                             cudaStream_t st) {
         const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
@@ -85,14 +94,14 @@ struct Launch {
             }
             if (pairs(g)) {
                 const Shape sp = shape_pairs(g, pair_threads<Q>());
-                k_step_pull2<Q, S, false><<<sp.grid, sp.block, 0, st>>>(g, cf, VelField<float>{}, a, b, flag);
+                LBM_EARLY(k_step_pull2, (Q, S, false, false), sp.grid, sp.block, g, cf, VelField<float>{}, a, b, flag);
                 return cudaGetLastError();
             }
         }
         if (g.link)
-            k_step_pull<Q, S, true><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+            LBM_EARLY(k_step_pull, (Q, S, true), sh.grid, sh.block, g, cf, a, b, flag);
         else
-            k_step_pull<Q, S, false><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+            LBM_EARLY(k_step_pull, (Q, S, false), sh.grid, sh.block, g, cf, a, b, flag);
         return cudaGetLastError();
     }
 
@@ -117,22 +126,23 @@ struct Launch {
             if (pairs(g)) {
                 const Shape sp = shape_pairs(g, pair_threads<Q>());
                 if (odd)
-                    k_step_aa_odd2<Q, S><<<sp.grid, sp.block, 0, st>>>(g, cf, VelField<float>{}, a, b, flag);
+                    LBM_EARLY(k_step_aa_odd2, (Q, S, false), sp.grid, sp.block, g, cf, VelField<float>{}, a, b, flag);
                 else
-                    k_step_aa_even2<Q, S, false><<<sp.grid, sp.block, 0, st>>>(g, cf, VelField<float>{}, a, b, flag);
+                    LBM_EARLY(k_step_aa_even2, (Q, S, false, false), sp.grid, sp.block, g, cf, VelField<float>{}, a,
+                              b, flag);
                 return cudaGetLastError();
             }
         }
         if (g.link) {
             if (odd)
-                k_step_aa<Q, S, true, 1><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+                LBM_EARLY(k_step_aa, (Q, S, true, 1), sh.grid, sh.block, g, cf, a, b, flag);
             else
-                k_step_aa<Q, S, true, 0><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+                LBM_EARLY(k_step_aa, (Q, S, true, 0), sh.grid, sh.block, g, cf, a, b, flag);
         } else {
             if (odd)
-                k_step_aa<Q, S, false, 1><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+                LBM_EARLY(k_step_aa, (Q, S, false, 1), sh.grid, sh.block, g, cf, a, b, flag);
             else
-                k_step_aa<Q, S, false, 0><<<sh.grid, sh.block, 0, st>>>(g, cf, a, b, flag);
+                LBM_EARLY(k_step_aa, (Q, S, false, 0), sh.grid, sh.block, g, cf, a, b, flag);
         }
         return cudaGetLastError();
     }
@@ -174,12 +184,26 @@ struct Launch {
             else K<Q, S, false, LAYOUT_LOCAL><<<sh.grid, sh.block, 0, st>>>(__VA_ARGS__);          \
         }                                                                                          \
     } while (0)
+#define LBM_BY_LAYOUT_EARLY(K, ...)                                                                \
+    do {                                                                                           \
+        const bool m_ = g.link != nullptr;                                                         \
+        if (layout == LAYOUT_PULL) {                                                               \
+            if (m_) LBM_EARLY(K, (Q, S, true, LAYOUT_PULL), sh.grid, sh.block, __VA_ARGS__);       \
+            else LBM_EARLY(K, (Q, S, false, LAYOUT_PULL), sh.grid, sh.block, __VA_ARGS__);         \
+        } else if (layout == LAYOUT_AAODD) {                                                       \
+            if (m_) LBM_EARLY(K, (Q, S, true, LAYOUT_AAODD), sh.grid, sh.block, __VA_ARGS__);      \
+            else LBM_EARLY(K, (Q, S, false, LAYOUT_AAODD), sh.grid, sh.block, __VA_ARGS__);        \
+        } else {                                                                                   \
+            if (m_) LBM_EARLY(K, (Q, S, true, LAYOUT_LOCAL), sh.grid, sh.block, __VA_ARGS__);      \
+            else LBM_EARLY(K, (Q, S, false, LAYOUT_LOCAL), sh.grid, sh.block, __VA_ARGS__);        \
+        }                                                                                          \
+    } while (0)
 
     static cudaError_t moments(const Geom& g, const void* coef, int layout, const void* src, void* rho, void* u,
                                void* Pi, void* f, cudaStream_t st) {
         const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
         const CF& cf = *static_cast<const CF*>(coef);
-        LBM_BY_LAYOUT(k_moments, g, cf, cpl(src, g), static_cast<T*>(rho), static_cast<T*>(u),
+        LBM_BY_LAYOUT_EARLY(k_moments, g, cf, cpl(src, g), static_cast<T*>(rho), static_cast<T*>(u),
                       static_cast<T*>(Pi), static_cast<T*>(f));
         return cudaGetLastError();
     }
@@ -220,10 +244,11 @@ struct Launch {
                 return cudaGetLastError();
             }
         }
-        LBM_BY_LAYOUT(k_adj_step, g, cf, cpl(src, g), cfl(lam_next, g), mfl(lam, g), gpart);
+        LBM_BY_LAYOUT_EARLY(k_adj_step, g, cf, cpl(src, g), cfl(lam_next, g), mfl(lam, g), gpart);
         return cudaGetLastError();
     }
 #undef LBM_BY_LAYOUT
+#undef LBM_BY_LAYOUT_EARLY
 
     static cudaError_t adj_init(const Geom& g, const void* coef, const void* rho0, const void* u0, const void* lam0,
                                 void* du0, double* gpart, cudaStream_t st) {
@@ -262,15 +287,17 @@ struct Launch {
             }
             if (pairs(g)) {
                 const Shape sp = shape_pairs(g, pair_threads<Q>());
-                k_step_pull2<Q, S, false, true><<<sp.grid, sp.block, 0, st>>>(g, cf, vel_field(u, g), cpl(src, g),
-                                                                            mpl(dst, g), flag);
+                LBM_EARLY(k_step_pull2, (Q, S, false, true), sp.grid, sp.block, g, cf, vel_field(u, g), cpl(src, g),
+                          mpl(dst, g), flag);
                 return cudaGetLastError();
             }
         }
         if (g.link)
-            k_ade_pull<Q, S, true><<<sh.grid, sh.block, 0, st>>>(g, cf, vel_field(u, g), cpl(src, g), mpl(dst, g), flag);
+            LBM_EARLY(k_ade_pull, (Q, S, true), sh.grid, sh.block, g, cf, vel_field(u, g), cpl(src, g), mpl(dst, g),
+                      flag);
         else
-            k_ade_pull<Q, S, false><<<sh.grid, sh.block, 0, st>>>(g, cf, vel_field(u, g), cpl(src, g), mpl(dst, g), flag);
+            LBM_EARLY(k_ade_pull, (Q, S, false), sh.grid, sh.block, g, cf, vel_field(u, g), cpl(src, g), mpl(dst, g),
+                      flag);
         return cudaGetLastError();
     }
 
@@ -295,22 +322,22 @@ struct Launch {
             if (pairs(g)) {
                 const Shape sp = shape_pairs(g, pair_threads<Q>());
                 if (odd)
-                    k_step_aa_odd2<Q, S, true><<<sp.grid, sp.block, 0, st>>>(g, cf, v, a, b, flag);
+                    LBM_EARLY(k_step_aa_odd2, (Q, S, true), sp.grid, sp.block, g, cf, v, a, b, flag);
                 else
-                    k_step_aa_even2<Q, S, false, true><<<sp.grid, sp.block, 0, st>>>(g, cf, v, a, b, flag);
+                    LBM_EARLY(k_step_aa_even2, (Q, S, false, true), sp.grid, sp.block, g, cf, v, a, b, flag);
                 return cudaGetLastError();
             }
         }
         if (g.link) {
             if (odd)
-                k_ade_aa<Q, S, true, 1><<<sh.grid, sh.block, 0, st>>>(g, cf, v, a, b, flag);
+                LBM_EARLY(k_ade_aa, (Q, S, true, 1), sh.grid, sh.block, g, cf, v, a, b, flag);
             else
-                k_ade_aa<Q, S, true, 0><<<sh.grid, sh.block, 0, st>>>(g, cf, v, a, b, flag);
+                LBM_EARLY(k_ade_aa, (Q, S, true, 0), sh.grid, sh.block, g, cf, v, a, b, flag);
         } else {
             if (odd)
-                k_ade_aa<Q, S, false, 1><<<sh.grid, sh.block, 0, st>>>(g, cf, v, a, b, flag);
+                LBM_EARLY(k_ade_aa, (Q, S, false, 1), sh.grid, sh.block, g, cf, v, a, b, flag);
             else
-                k_ade_aa<Q, S, false, 0><<<sh.grid, sh.block, 0, st>>>(g, cf, v, a, b, flag);
+                LBM_EARLY(k_ade_aa, (Q, S, false, 0), sh.grid, sh.block, g, cf, v, a, b, flag);
         }
         return cudaGetLastError();
     }

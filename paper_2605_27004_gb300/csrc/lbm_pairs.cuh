@@ -230,15 +230,15 @@ __device__ __forceinline__ bool bad1(float rho, float ux, float uy, float uz) {
 // Collision of the pair at cell index n (even): the flow's BGK, or (ADE) the advection-diffusion
 // relaxation of a scalar with the prescribed velocity read as one aligned vector per component
 // (lbm_ade.cuh). Returns true when a fluid cell of the pair (fa, fb) is unstable.
-template <int Q, int S, bool ADE>
+template <int Q, int S, bool ADE, bool EARLY = false>
 __device__ __forceinline__ bool collide2(const Coef<float>& cf, const VelField<float>& vf, uint32_t n, F2 (&d)[Q],
                                          bool fa, bool fb) {
     if constexpr (ADE) {
         F2 ux = f2(0.f), uy = f2(0.f), uz = f2(0.f);
         if (vf.p[0] != nullptr) {
-            ux = ld2(vf.p[0] + n);
-            uy = ld2(vf.p[1] + n);
-            if (Lat<Q>::D == 3) uz = ld2(vf.p[2] + n);
+            ux = EARLY ? ld2_rw(vf.p[0] + n) : ld2(vf.p[0] + n);
+            uy = EARLY ? ld2_rw(vf.p[1] + n) : ld2(vf.p[1] + n);
+            if (Lat<Q>::D == 3) uz = EARLY ? ld2_rw(vf.p[2] + n) : ld2(vf.p[2] + n);
         }
         F2 s = d[0];
 #pragma unroll
@@ -264,12 +264,13 @@ constexpr int pair_threads() {
     return Q == 27 ? 128 : 256;
 }
 
-template <int Q, int S, bool MASK, bool ADE = false>
+template <int Q, int S, bool MASK, bool ADE, bool EARLY>
 __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 : 3))
     k_step_pull2(Geom g, Coef<float> cf, VelField<float> vf, const Planes<const typename Store<S>::type> src,
                  const Planes<typename Store<S>::type> dst, int* __restrict__ flag) {
     PCell c;
     make_pcell(g, c);
+    wait_previous<EARLY>();
     uint2 lw = make_uint2(0u, 0u);
     if (MASK && c.in_grid) lw = __ldg(reinterpret_cast<const uint2*>(g.link + c.n));
     const bool fa = !(lw.x & LINK_SOLID), fb = !(lw.y & LINK_SOLID);
@@ -278,17 +279,17 @@ __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 :
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const Vec3 v = vel<Q>(i);
-        d[i] = gather_pair<S, true>(src.p[i], c.R[v.y + 1][v.z + 1], c, v.x, g.nx, cf.so[i]);
+        d[i] = gather_pair<S, !EARLY>(src.p[i], c.R[v.y + 1][v.z + 1], c, v.x, g.nx, cf.so[i]);
         if (MASK && i > 0) {
             const bool wa = link_bit(lw.x, i), wb = link_bit(lw.y, i);
             if (c.active && (wa || wb)) {  // half-way bounce-back from the own cell's opposite slot
-                const F2 own = to_shifted2<S>(ld2(src.p[opp(i)] + c.n), cf.so[i]);
+                const F2 own = to_shifted2<S>(EARLY ? ld2_rw(src.p[opp(i)] + c.n) : ld2(src.p[opp(i)] + c.n), cf.so[i]);
                 d[i] = f2(wa ? own.v.x : d[i].v.x, wb ? own.v.y : d[i].v.y);
             }
         }
     }
     if (!c.active) return;
-    if (collide2<Q, S, ADE>(cf, vf, c.n, d, fa, fb)) *flag = 1;
+    if (collide2<Q, S, ADE, EARLY>(cf, vf, c.n, d, fa, fb)) *flag = 1;
     if (!MASK || (fa && fb)) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) st2(dst.p[i] + c.n, from_shifted2<S>(d[i], cf.so[i]));
@@ -305,12 +306,13 @@ __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 :
 // ---------------------------------------------------------------------------------------------
 // AA even step (state LOCAL -> AAODD), two cells per thread: purely local.
 // ---------------------------------------------------------------------------------------------
-template <int Q, int S, bool MASK, bool ADE = false>
+template <int Q, int S, bool MASK, bool ADE, bool EARLY>
 __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 : 3))
     k_step_aa_even2(Geom g, Coef<float> cf, VelField<float> vf, const Planes<const typename Store<S>::type> src,
                     const Planes<typename Store<S>::type> dst, int* __restrict__ flag) {
     PCell c;
     make_pcell(g, c);
+    wait_previous<EARLY>();
     if (!c.in_grid) return;
     uint2 lw = make_uint2(0u, 0u);
     if (MASK) lw = __ldg(reinterpret_cast<const uint2*>(g.link + c.n));
@@ -319,7 +321,7 @@ __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 :
     F2 d[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) d[i] = to_shifted2<S>(ld2_rw(src.p[i] + c.n), cf.so[i]);
-    if (collide2<Q, S, ADE>(cf, vf, c.n, d, fa, fb)) *flag = 1;
+    if (collide2<Q, S, ADE, EARLY>(cf, vf, c.n, d, fa, fb)) *flag = 1;
     if (!MASK || (fa && fb)) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) st2(dst.p[opp(i)] + c.n, from_shifted2<S>(d[i], cf.so[i]));
@@ -344,12 +346,13 @@ __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 :
 // vector loads may also fetch an element that another thread consumes and replaces; such an
 // element is never used by the fetching thread.)
 // ---------------------------------------------------------------------------------------------
-template <int Q, int S, bool ADE = false>
+template <int Q, int S, bool ADE, bool EARLY>
 __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 : 3))
     k_step_aa_odd2(Geom g, Coef<float> cf, VelField<float> vf, const Planes<const typename Store<S>::type> src,
                    const Planes<typename Store<S>::type> dst, int* __restrict__ flag) {
     PCell c;
     make_pcell(g, c);
+    wait_previous<EARLY>();
     c.active = c.in_grid;
     F2 d[Q];
 #pragma unroll
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(pair_threads<Q>(), Q == 27 ? 5 : (S != 3 ? 2 :
         const Vec3 v = vel<Q>(i);
         d[i] = gather_pair<S, false>(src.p[opp(i)], c.R[v.y + 1][v.z + 1], c, v.x, g.nx, cf.so[i]);
     }
-    if (c.active && collide2<Q, S, ADE>(cf, vf, c.n, d, true, true)) *flag = 1;
+    if (c.active && collide2<Q, S, ADE, EARLY>(cf, vf, c.n, d, true, true)) *flag = 1;
     const int nx = g.nx;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
