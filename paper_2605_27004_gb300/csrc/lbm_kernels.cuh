@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S
 // Each thread writes exactly the slots it read, so the in-place update is race free. The link
 // bit of x + c_i is the bit of direction opp(i).
 // ---------------------------------------------------------------------------------------------
-template <int Q, int S, bool MASK, int ODD>
+template <int Q, int S, bool MASK, int ODD, bool RAW = false>
 __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<typename Store<S>::T>& cf,
                                          const Planes<typename Store<S>::type>& dst,
                                          const typename Store<S>::T (&d)[Q]) {
@@ -565,7 +565,7 @@ __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<
             else
                 p = dst.p[i] + off_plus(c, v);
         }
-        st_raw(p, stored<S>(d[i], cf.so[i]));
+        st_raw(p, RAW ? d[i] : from_shifted<S>(d[i], cf.so[i]));
     }
 }
 
@@ -595,9 +595,9 @@ __global__ void __launch_bounds__(256) k_step_aa(Geom g, Coef<typename Store<S>:
     const Macro<T> m = collide<Q, S>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
-        aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);
+        aa_store<Q, S, false, ODD, S == 1>(c, 0u, cf, dst, d);
     else
-        aa_store<Q, S, MASK, ODD>(c, lw, cf, dst, d);
+        aa_store<Q, S, MASK, ODD, S == 1>(c, lw, cf, dst, d);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -707,9 +707,9 @@ __global__ void __launch_bounds__(256, 4) k_step_aa_list(Geom g, Coef<typename S
     const Macro<T> m = collide<Q, S>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
-        aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);
+        aa_store<Q, S, false, ODD, S == 1>(c, 0u, cf, dst, d);
     else
-        aa_store<Q, S, true, ODD>(c, lw, cf, dst, d);
+        aa_store<Q, S, true, ODD, S == 1>(c, lw, cf, dst, d);
 }
 
 // ---------------------------------------------------------------------------------------------
