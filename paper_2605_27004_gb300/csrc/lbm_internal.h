@@ -139,6 +139,9 @@ struct Ops {
     // the scalar pull step over the sector list (boxes with walls, FP16 and FP32 storage)
     cudaError_t (*ade_pull_sectors)(const Geom&, const void* coef, const CellList&, const void* u, const void* src,
                                     void* dst, int* flag, cudaStream_t);
+    // two flow steps of the pull scheme in one launch (lbm_twice.cuh), for the boxes `twice` accepts
+    bool (*twice)(const Geom&);
+    cudaError_t (*step_twice)(const Geom&, const void* coef, const void* src, void* dst, int* flag, cudaStream_t);
 };
 
 // One translation unit per (lattice, storage): lbm_ops.cu compiled with LBM_Q / LBM_S, and for

@@ -1,11 +1,13 @@
 // Host-side launchers of one (lattice, storage) pair: kernel choice (one or two cells per
 // thread), launch shapes and the dispatch over walls and layouts.
 #pragma once
+#include <algorithm>
 #include "lbm_ade.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_adjoint2.cuh"
 #include "lbm_pairs.cuh"
 #include "lbm_quads.cuh"
+#include "lbm_twice.cuh"
 
 namespace lbm {
 inline namespace LBM_VARIANT {
@@ -352,10 +354,42 @@ struct Launch {
         return cudaGetLastError();
     }
 
+    // FP32 storage on D3Q19 in whole boxes (lbm_twice.cuh)
+    static constexpr bool TWICE = (S == 0 || S == 2) && Q == 19 && !LBM_SLAB;
+    static int sm_count() {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        return sms;
+    }
+    static bool twice(const Geom& g) {
+        if constexpr (TWICE) return !g.link && twice_pays(g, sm_count());
+        return false;
+    }
+
+    static cudaError_t step_twice(const Geom& g, const void* coef, const void* src, void* dst, int* flag,
+                                  cudaStream_t st) {
+        if constexpr (TWICE) {
+            long long walks = 0;
+            const Tiles t = twice_tiles(g, std::max(1, sm_count()), walks);
+            const cudaError_t e = cudaFuncSetAttribute(k_step_twice<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       twice_smem<Q>());
+            if (e != cudaSuccess) return e;
+            const long long n = t.chunks ? (long long)t.tiles * t.chunks : ((long long)t.tiles * g.nz + t.run - 1) / t.run;
+            k_step_twice<Q, S><<<(unsigned)n, TWICE_THREADS, twice_smem<Q>(), st>>>(
+                g, *static_cast<const CF*>(coef), t, cpl(src, g), mpl(dst, g), flag);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
+    }
+
     static const Ops& ops() {
         static const Ops o = {&init,     &step_pull, &step_aa,   &step_pull_sectors, &step_aa_list, &moments,
                               &totals,   &adj_seed,  &adj_step,  &adj_init,          &link_mask,    &ade_pull,
-                              &ade_aa,   &ade_pull_sectors};
+                              &ade_aa,   &ade_pull_sectors, &twice, &step_twice};
         return o;
     }
 };

@@ -21,3 +21,34 @@ def test_fp64_step_block_edges(q, dims, scheme):
     g = gpu_run(q, dims, 0.8, Th, rho0, u0, 20, storage="fp64", scheme=scheme)
     o = oracle_run(q, dims, 0.8, Th, rho0, u0, 20)
     assert np.abs(g["f"] - o["f"][:, perm_lib_to_oracle(q)].T).max() < 1e-13
+
+
+# D3Q19 FP32 boxes run two steps per launch: the same arithmetic, so the same bits as single steps.
+# Tiles of 64 x 9 cells: rows in one, two and three tiles (the last narrower), rows left over in y,
+# planes split among blocks in chunks of one tile and in runs over several; odd step counts, and
+# stops for a check and for recorded checkpoints inside the run; boxes on both sides of the rule that
+# takes them there.
+@pytest.mark.parametrize("storage", ["fp32s", "fp32"])
+@pytest.mark.parametrize("dims,pays", [((128, 128, 128), True), ((64, 180, 181), True), ((120, 130, 140), True),
+                                       ((192, 99, 160), True), ((192, 100, 113), False), ((8, 1, 1), False)])
+def test_two_steps_per_launch_match_single_steps(dims, pays, storage):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    N = int(np.prod(dims))
+    Th = rand_theta(3, 3)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rho = 1 + 0.02 * torch.randn(N, device="cuda", generator=g)
+    u = 0.03 * torch.randn(3, N, device="cuda", generator=g)
+    runs = []
+    for together, kw in ((True, {}), (False, {}), (True, {"check_every": 5}), (True, {"use_graphs": 1})):
+        L = lbm.LBM(19, *dims, 0.62, Th, storage=storage, **kw)
+        L.record_checkpoints(7 if kw else 0)
+        L.init(rho, u)
+        before = L.launches
+        for n in [17] if together else [1] * 17:
+            L.step(n)
+        runs.append((L.launches - before, L.populations()))
+    assert runs[1][0] == 17
+    assert runs[0][0] == (9 if pays else 17)
+    for _, f in runs:
+        assert torch.equal(f, runs[1][1])
