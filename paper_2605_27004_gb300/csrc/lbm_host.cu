@@ -74,6 +74,17 @@ __global__ void __launch_bounds__(256) k_halo_copy(E* __restrict__ arr, E* __res
     }
 }
 
+// The link words of the listed cells in list order: entry k stands for the cells G idx[k] .. + G - 1.
+__global__ void __launch_bounds__(256) k_list_links(const uint32_t* __restrict__ idx, unsigned long long count, uint32_t G,
+                                                    uint32_t N, const uint32_t* __restrict__ link,
+                                                    uint32_t* __restrict__ out) {
+    for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < count * G;
+         t += (unsigned long long)gridDim.x * blockDim.x) {
+        const uint32_t n = idx[t / G] * G + (uint32_t)(t % G);
+        out[t] = n < N ? link[n] : LINK_SOLID;
+    }
+}
+
 template <typename T>
 __global__ void k_fill(T* __restrict__ p, long long n, T v) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -137,6 +148,10 @@ struct lbm_ctx {
     long long n_fluid = 0;
     uint32_t* cell_idx = nullptr;  // with walls: fluid cells (FP16 AA) or 32-byte sectors (FP16 / FP32 pull)
     CellList cells{};
+    uint32_t* cell_link = nullptr;  // their link words
+    size_t cell_link_bytes = 0;
+    uint2* sectors = nullptr;  // with walls, FP16 AA: the even step's sectors
+    SectorList sector_list{};
 
     Coef<double> cd{};
     Coef<float> cf{};
@@ -337,9 +352,22 @@ void drop_graph(lbm_ctx* c) {
     c->graph_steps = 0;
 }
 
+void drop_lists(lbm_ctx* c) {
+    dev_free(c, c->cell_idx, (size_t)c->cells.count * 4 + 4);
+    dev_free(c, c->cell_link, c->cell_link_bytes);
+    dev_free(c, c->sectors, (size_t)c->sector_list.count * 8 + 8);
+    c->cell_idx = c->cell_link = nullptr;
+    c->sectors = nullptr;
+    c->cell_link_bytes = 0;
+    c->cells = CellList{};
+    c->sector_list = SectorList{};
+}
+
 // One forward step src -> dst of a flow context on stream s (t = steps done before it): over the
 // lists of a context with walls (sectors for pull, cells for FP16 AA), else over the grid.
 cudaError_t step_kernel(lbm_ctx* c, const void* src, void* dst, long long t, cudaStream_t s) {
+    if (c->sectors && (t & 1) == 0)
+        return c->ops->step_aa_even_sectors(c->geom, c->coef(), c->sector_list, src, dst, c->flag, s);
     if (c->cell_idx)
         return c->scheme == LBM_PULL2
                    ? c->ops->step_pull_sectors(c->geom, c->coef(), c->cells, src, dst, c->flag, s)
@@ -645,7 +673,7 @@ void lbm_destroy(lbm_ctx* c) {
     dev_free(c, c->pop[0], SB);
     dev_free(c, c->pop[1], SB);
     dev_free(c, c->link, (size_t)c->N * 4);
-    dev_free(c, c->cell_idx, (size_t)c->cells.count * 4 + 4);
+    drop_lists(c);
     for (size_t k = 0; k < c->rec_ptr.size(); ++k) {
         if (!c->rec_ptr[k]) continue;
         if (c->rec_host[k])
@@ -800,11 +828,38 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
                 e = cudaMemcpy(c->cell_idx, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice);
                 if (e != cudaSuccess) return bail(cuda_fail(c, e, "fluid-cell list upload"));
                 c->cells.idx = c->cell_idx;
+                const uint32_t G = c->scheme == LBM_AA ? 1 : fp16 ? 16 : 8;  // cells of an entry
+                c->cell_link_bytes = idx.size() * G * 4 + 4;
+                c->cell_link = (uint32_t*)dev_alloc(c, c->cell_link_bytes);
+                if (!c->cell_link) return bail(fail(c, LBM_ERR_OOM, "listed link words"));
+                c->cells.link = c->cell_link;
+                if (!idx.empty()) {
+                    const unsigned long long total = idx.size() * (unsigned long long)G;
+                    k_list_links<<<(unsigned)std::min<unsigned long long>((total + 255) / 256, 8 * 152), 256, 0, c->stream>>>(
+                        c->cell_idx, idx.size(), G, c->geom.N, c->link, c->cell_link);
+                    e = cudaGetLastError();
+                    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+                    if (e != cudaSuccess) return bail(cuda_fail(c, e, "listed link words"));
+                }
                 c->cells.count = (uint32_t)idx.size();
                 c->cells.rnx = ~0ULL / (unsigned long long)nx + 1ULL;
                 c->cells.rnxy = ~0ULL / (unsigned long long)plane + 1ULL;
                 c->cells.n_begin = (uint32_t)nb;
                 c->cells.n_end = (uint32_t)ne;
+                if (c->scheme == LBM_AA && c->storage == LBM_FP16_SHIFTED && c->kind == 0 && c->N % 2 == 0) {
+                    std::vector<uint2> sec;
+                    for (long long n0 = 0; n0 < c->N; n0 += 16) {
+                        uint32_t bits = 0;
+                        for (long long n = n0; n < std::min(n0 + 16, c->N); ++n) bits |= (m[(size_t)n] ? 0u : 1u) << (n - n0);
+                        if (bits) sec.push_back(make_uint2((uint32_t)(n0 / 16), bits));
+                    }
+                    c->sectors = (uint2*)dev_alloc(c, sec.size() * 8 + 8);
+                    if (!c->sectors) return bail(fail(c, LBM_ERR_OOM, "sector list"));
+                    c->sector_list.count = (uint32_t)sec.size();
+                    e = cudaMemcpy(c->sectors, sec.data(), sec.size() * 8, cudaMemcpyHostToDevice);
+                    if (e != cudaSuccess) return bail(cuda_fail(c, e, "sector list upload"));
+                    c->sector_list.sector = c->sectors;
+                }
             }
         }
     }
@@ -1516,11 +1571,7 @@ int lbm_ade_create(lbm_ctx** out, int lattice, int nx, int ny, int nz, double ta
     if (rc == LBM_OK) {
         lbm_ctx* c = *out;
         c->kind = 1;
-        if (c->scheme != LBM_PULL2) {  // the scalar's AA steps run over the grid: no fluid-cell list
-            dev_free(c, c->cell_idx, (size_t)c->cells.count * 4 + 4);
-            c->cell_idx = nullptr;
-            c->cells = CellList{};
-        }
+        if (c->scheme != LBM_PULL2) drop_lists(c);  // the scalar's AA steps run over the grid
     }
     return rc;
 }

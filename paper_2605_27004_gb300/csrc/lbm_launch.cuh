@@ -67,6 +67,13 @@ struct Launch {
     // populations per thread and stays at two cells.
     static bool quads(const Geom& g) { return S == 3 && Q != 27 && !g.link && (g.nx % 128) == 0; }
 
+    // Rows of odd length, FP16 storage without walls: two cells of a row per thread (lbm_cells2.cuh).
+    static bool odd_rows(const Geom& g) { return S == 3 && !g.link && (g.nx % 2) == 1 && g.nx >= 3; }
+    static unsigned blocks_rows2(const Geom& g) {
+        const unsigned long long t = (unsigned long long)((g.nx + 1) / 2) * g.ny * (g.nz - 2 * LBM_SLAB);
+        return (unsigned)((t + CELLS2_THREADS - 1) / CELLS2_THREADS);
+    }
+
     // FP64 steps are bound by the FP64 pipes, so their blocks have 64 threads: a small box then
     // reaches every SM (64^2 ran on 16 of them: 11.2 -> 4.6 us a step with the FP64 collision of
     // bgk_raw; 33 x 29 x 41 37.3 -> 29.5 us against 256 threads; from 64^3 up there is no
@@ -97,6 +104,10 @@ struct Launch {
             if (pairs(g)) {
                 const Shape sp = shape_pairs(g, pair_threads<Q>());
                 LBM_EARLY(k_step_pull2, (Q, S, false, false), sp.grid, sp.block, g, cf, VelField<float>{}, a, b, flag);
+                return cudaGetLastError();
+            }
+            if (odd_rows(g)) {
+                LBM_EARLY(k_step_pull_rows2, (Q), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
                 return cudaGetLastError();
             }
         }
@@ -132,6 +143,13 @@ struct Launch {
                 else
                     LBM_EARLY(k_step_aa_even2, (Q, S, false, false), sp.grid, sp.block, g, cf, VelField<float>{}, a,
                               b, flag);
+                return cudaGetLastError();
+            }
+            if (odd_rows(g)) {
+                if (odd)
+                    LBM_EARLY(k_step_aa_rows2, (Q, 1), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
+                else
+                    LBM_EARLY(k_step_aa_rows2, (Q, 0), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
                 return cudaGetLastError();
             }
         }
@@ -386,10 +404,22 @@ struct Launch {
         return cudaErrorNotSupported;
     }
 
+    static cudaError_t step_aa_even_sectors(const Geom& g, const void* coef, const SectorList& L, const void* src,
+                                            void* dst, int* flag, cudaStream_t st) {
+        if constexpr (S == 3) {
+            if (L.count == 0) return cudaSuccess;
+            const unsigned nb = (unsigned)((L.count * 8ull + CELLS2_THREADS - 1) / CELLS2_THREADS);
+            k_step_aa_even_sectors2<Q><<<nb, CELLS2_THREADS, 0, st>>>(g, *static_cast<const CF*>(coef), L, cpl(src, g),
+                                                                     mpl(dst, g), flag);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
+    }
+
     static const Ops& ops() {
         static const Ops o = {&init,     &step_pull, &step_aa,   &step_pull_sectors, &step_aa_list, &moments,
                               &totals,   &adj_seed,  &adj_step,  &adj_init,          &link_mask,    &ade_pull,
-                              &ade_aa,   &ade_pull_sectors, &twice, &step_twice};
+                              &ade_aa,   &ade_pull_sectors, &step_aa_even_sectors, &twice, &step_twice};
         return o;
     }
 };

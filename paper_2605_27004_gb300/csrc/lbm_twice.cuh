@@ -25,67 +25,10 @@
 // The arithmetic is that of the one-cell kernels operation for operation (collide_pair), so that two
 // steps in one launch give the bits of two launches.
 #pragma once
-#include "lbm_pairs.cuh"
+#include "lbm_cells2.cuh"
 
 namespace lbm {
 inline namespace LBM_VARIANT {
-
-// bgk<Q, float, true, false> on two cells, in the order of operations (fused multiply-adds included)
-// that the one-cell kernels are compiled to; tests/test_gpu_step_paths.py holds the two bit for bit.
-template <int Q>
-__device__ __forceinline__ Macro2 collide_pair(const Coef<float>& cf, F2 (&d)[Q]) {
-    Macro2 m;
-    F2 s = d[0], jx = f2(0.f), jy = f2(0.f), jz = f2(0.f);
-#pragma unroll
-    for (int k = 0; k < Lat<Q>::P; ++k) {
-        const F2 a = d[2 * k + 1], b = d[2 * k + 2];
-        s += a + b;
-        add_c2(vel<Q>(2 * k + 1), a - b, jx, jy, jz);
-    }
-    m.drho = s;
-    m.rho = f2(cf.rho0) + s;
-    m.jx = jx;
-    m.jy = jy;
-    m.jz = jz;
-    const F2 inv = f2(1.f / m.rho.v.x, 1.f / m.rho.v.y);
-    m.ux = jx * inv;
-    m.uy = jy * inv;
-    m.uz = jz * inv;
-    const F2 usq = fma2(m.uz, m.uz, fma2(m.ux, m.ux, m.uy * m.uy));
-    const F2 nusq = -usq, nusq3 = -(usq * f2(1.0f / 3.0f));
-    // -2 K~.u
-    const F2 kx = f2(-2.f) * fma2(f2(cf.K[4]), m.uz, fma2(f2(cf.K[0]), m.ux, f2(cf.K[3]) * m.uy));
-    const F2 ky = f2(-2.f) * fma2(f2(cf.K[5]), m.uz, fma2(f2(cf.K[3]), m.ux, f2(cf.K[1]) * m.uy));
-    const F2 kz = f2(-2.f) * fma2(f2(cf.K[2]), m.uz, fma2(f2(cf.K[5]), m.uy, f2(cf.K[4]) * m.ux));
-    const F2 r45 = f2(4.5f) * m.rho, nrho = -m.rho;
-    const F2 om = f2(cf.omega), om1 = f2(1.f - cf.omega);
-    const F2 rest = fma2(s, f2(cf.A[0]), f2((float)weight<Q>(0)) * r45 * usq * f2(-1.0f / 3.0f));
-    d[0] = fma2(om1, d[0], om * rest);
-    F2 ex = -jx, ey = -jy, ez = -jz;  // post-collision momentum defect
-#pragma unroll
-    for (int k = 0; k < Lat<Q>::P; ++k) {
-        const int i = 2 * k + 1;
-        const Vec3 v = vel<Q>(i);
-        const float w = (float)weight<Q>(i);
-        const F2 uc = vdot2(v, m.ux, m.uy, m.uz);
-        const F2 nqk2 = vdot2(v, kx, ky, kz);
-        const F2 E = fma2(s, f2(cf.A[i]), (f2(w) * r45) * fma2(uc, uc, nusq3));
-        const F2 H = fma2(uc, fma2(uc, uc, nusq), nqk2);
-        const F2 J = fma2(uc, f2(cf.B[i]), f2(w * cf.c3) * H);
-        d[i] = fma2(om1, d[i], om * fma2(m.rho, J, E));
-        d[i + 1] = fma2(om1, d[i + 1], om * fma2(nrho, J, E));
-        add_c2(v, d[i] - d[i + 1], ex, ey, ez);
-    }
-#pragma unroll
-    for (int k = 0; k < Lat<Q>::P; ++k) {
-        const Vec3 v = vel<Q>(2 * k + 1);
-        const float c = (float)(3.0 * weight<Q>(2 * k + 1));
-        const F2 e = vdot2(v, ex, ey, ez);
-        d[2 * k + 1] = fma2(f2(-c), e, d[2 * k + 1]);
-        d[2 * k + 2] = fma2(f2(c), e, d[2 * k + 2]);
-    }
-    return m;
-}
 
 constexpr int TWICE_ROWS = 11;        // rows of a block's ring-extended tile
 constexpr int TWICE_W = 64;           // cells of a row of the tile, at most
@@ -200,7 +143,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
                 F2 d[Q];
 #pragma unroll
                 for (int i = 0; i < Q; ++i) d[i] = to_shifted2<S>(e[i], cf.so[i]);
-                const Macro2 m = collide_pair<Q>(cf, d);
+                const Macro2 m = collide_pair<Q, S>(cf, d);
                 bad |= bad1(m.rho.v.x, m.ux.v.x, m.uy.v.x, m.uz.v.x) || bad1(m.rho.v.y, m.ux.v.y, m.uy.v.y, m.uz.v.y);
                 float* o = sh + r * P;
                 float* of = o + b2 * (twice_count<Q>(0) * RP);
@@ -238,7 +181,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
                     else
                         d[i] = to_shifted2<S>(f2(q[0], q[second]), cf.so[i]);
                 }
-                const Macro2 m = collide_pair<Q>(cf, d);
+                const Macro2 m = collide_pair<Q, S>(cf, d);
                 bad |= bad1(m.rho.v.x, m.ux.v.x, m.uy.v.x, m.uz.v.x) || bad1(m.rho.v.y, m.ux.v.y, m.uy.v.y, m.uz.v.y);
                 const uint32_t n = row_out + nxy * (uint32_t)(p - 1);
 #pragma unroll

@@ -52,3 +52,35 @@ def test_two_steps_per_launch_match_single_steps(dims, pays, storage):
     assert runs[0][0] == (9 if pays else 17)
     for _, f in runs:
         assert torch.equal(f, runs[1][1])
+
+
+# FP16 storage in rows of odd length, and AA with walls: two cells per thread. The FP16 form shifted by
+# the weights runs one cell per thread, and at Theta = cs2 I its stored values and its arithmetic
+# are the same, so the two give the same bits; so do pull and AA, which round the same post-collision
+# values. Rows of 3 to 67 cells (halves of one length and of two), boxes of an odd number of cells and
+# of a number that is no multiple of a sector's 16, boxes of one row and one plane.
+@pytest.mark.parametrize("q,dims,frac", [(9, (67, 9, 1), 0.0), (9, (3, 1, 1), 0.0), (19, (35, 4, 3), 0.0),
+                                         (27, (31, 3, 2), 0.0), (19, (5, 1, 7), 0.0), (9, (18, 9, 1), 0.2),
+                                         (19, (33, 4, 5), 0.2), (19, (7, 5, 3), 0.3), (27, (6, 5, 3), 0.3),
+                                         (27, (40, 6, 5), 0.5), (27, (16, 2, 1), 0.1)])
+def test_fp16_two_cells_match_one_cell(q, dims, frac):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    d, N = (2 if q == 9 else 3), int(np.prod(dims))
+    solid = inputs.random_mask(N, frac, 4) if frac else None
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rho = 1 + 0.02 * torch.randn(N, device="cuda", generator=g)
+    u = 0.03 * torch.randn(d, N, device="cuda", generator=g)
+
+    def run(storage, scheme, Th, steps):
+        L = lbm.LBM(q, *dims, 0.7, Th, storage=storage, scheme=scheme, solid=solid)
+        L.init(rho, u)
+        L.step(steps)
+        return L.populations()
+
+    iso = np.eye(d) / 3
+    for steps in (20, 21):
+        for scheme in ("pull", "aa"):
+            assert torch.equal(run("fp16s", scheme, iso, steps), run("fp16w", scheme, iso, steps))
+        Th = rand_theta(8, d)
+        assert torch.equal(run("fp16s", "pull", Th, steps), run("fp16s", "aa", Th, steps))
