@@ -195,6 +195,7 @@ struct lbm_ctx {
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     long long graph_launches = 0;  // kernels of one replay
+    bool graph_flips = false;      // a replay leaves the state in the other array
 
     // checkpoints recorded during the forward run (state at t = k * rec_K)
     int rec_K = 0;
@@ -407,23 +408,16 @@ cudaError_t launch_step(lbm_ctx* c, cudaStream_t s) {
     return e;
 }
 
-// Whether two steps may go into one launch (launch_steps with left >= 2).
-bool can_twice(const lbm_ctx* c) {
-    return c->kind == 0 && c->scheme == LBM_PULL2 && !c->slab && c->ops->twice(c->geom);
-}
-
-// One launch from the current state, of two steps where the context allows it and `left` does;
-// returns the steps taken in *taken.
-cudaError_t launch_steps(lbm_ctx* c, cudaStream_t s, long long left, bool twice, int* taken) {
-    if (!twice || left < 2) {
-        *taken = 1;
-        return launch_step(c, s);
-    }
-    const cudaError_t e = c->ops->step_twice(c->geom, c->coef(), c->pop[c->cur], c->pop[c->cur ^ 1], c->flag, s);
+// One launch from the current state: of several steps where the context allows it and `left` (the
+// steps to the next stop) does. Returns the steps taken in *taken.
+cudaError_t launch_steps(lbm_ctx* c, cudaStream_t s, long long left, int* taken) {
+    *taken = c->kind == 0 && c->scheme == LBM_PULL2 && !c->slab ? c->ops->steps_at_once(c->geom, left) : 1;
+    if (*taken == 1) return launch_step(c, s);
+    const cudaError_t e =
+        c->ops->step_several(c->geom, c->coef(), *taken, c->pop[c->cur], c->pop[c->cur ^ 1], c->flag, s);
     c->cur ^= 1;
-    c->steps += 2;
+    c->steps += *taken;
     c->launches += 1;
-    *taken = 2;
     return e;
 }
 
@@ -436,10 +430,10 @@ int ensure_graph(lbm_ctx* c, int gsteps) {
     const long long launches0 = c->launches;
     LBM_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
-    const bool twice = can_twice(c);
     for (int k = 0, taken = 0; k < gsteps && le == cudaSuccess; k += taken)
-        le = launch_steps(c, c->cap_stream, gsteps - k, twice, &taken);
+        le = launch_steps(c, c->cap_stream, gsteps - k, &taken);
     c->graph_launches = c->launches - launches0;
+    c->graph_flips = c->cur != cur0;
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
     c->cur = cur0;
@@ -954,7 +948,6 @@ int lbm_step(lbm_ctx* c, int n) {
     long long next_check = c->opt.check_every > 0 ? (c->steps / c->opt.check_every + 1) * c->opt.check_every : -1;
     const bool recording = c->rec_K > 0 && c->rec_valid * c->rec_K > c->steps;
     long long next_rec = recording ? (c->steps / c->rec_K + 1) * c->rec_K : -1;
-    const bool twice = n > 1 && can_twice(c);
     int left = n;
     while (left > 0) {
         const bool aligned = (c->steps & 1) == 0 && (c->scheme != LBM_PULL2 || c->cur == 0);
@@ -966,6 +959,7 @@ int lbm_step(lbm_ctx* c, int n) {
             LBM_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
             c->steps += gsteps;
             c->launches += c->graph_launches;
+            if (c->graph_flips) c->cur ^= 1;
             left -= gsteps;
             ran = true;
         }
@@ -974,7 +968,7 @@ int lbm_step(lbm_ctx* c, int n) {
             const long long stop = std::min(next_check < 0 ? c->steps + left : next_check,
                                             next_rec < 0 ? c->steps + left : next_rec);
             int taken = 0;
-            cudaError_t e = launch_steps(c, c->stream, std::min<long long>(left, stop - c->steps), twice, &taken);
+            cudaError_t e = launch_steps(c, c->stream, std::min<long long>(left, stop - c->steps), &taken);
             if (e != cudaSuccess) return cuda_fail(c, e, "stream-collide kernel");
             if (int rc = run_halo(c, LBM_HALO_POPULATIONS, state_ptr(c))) return rc;
             left -= taken;

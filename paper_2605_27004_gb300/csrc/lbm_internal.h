@@ -98,7 +98,7 @@ inline int block_x_for(int n, int threads = 256) {
 // Launch of a kernel that waits for the previous one itself (wait_previous) before its first access
 // to memory that another kernel writes: its blocks may be set up while that one drains.
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+cudaError_t launch_after_shared(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, size_t shared, A&&... args) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -106,11 +106,17 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.stream = st;
+    cfg.dynamicSmemBytes = shared;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... args) {
+    return launch_after_shared(kernel, grid, block, st, 0, static_cast<A&&>(args)...);
 }
 
 // Kernel launchers of one (lattice, storage) pair. `coef` points at a Coef<double> (storage
@@ -152,9 +158,11 @@ struct Ops {
     // the even AA step with walls over the sector list (FP16 r-shifted storage)
     cudaError_t (*step_aa_even_sectors)(const Geom&, const void* coef, const SectorList&, const void* src, void* dst,
                                         int* flag, cudaStream_t);
-    // two flow steps of the pull scheme in one launch (lbm_twice.cuh), for the boxes `twice` accepts
-    bool (*twice)(const Geom&);
-    cudaError_t (*step_twice)(const Geom&, const void* coef, const void* src, void* dst, int* flag, cudaStream_t);
+    // several flow steps of the pull scheme in one launch: `steps_at_once` says how many of `left` one
+    // launch takes (1: step_pull); src and dst are the two arrays, as for one step
+    int (*steps_at_once)(const Geom&, long long left);
+    cudaError_t (*step_several)(const Geom&, const void* coef, int steps, const void* src, void* dst, int* flag,
+                                cudaStream_t);
 };
 
 // One translation unit per (lattice, storage): lbm_ops.cu compiled with LBM_Q / LBM_S, and for

@@ -6,6 +6,7 @@
 #include "lbm_kernels.cuh"
 #include "lbm_adjoint2.cuh"
 #include "lbm_pairs.cuh"
+#include "lbm_plane.cuh"
 #include "lbm_quads.cuh"
 #include "lbm_twice.cuh"
 
@@ -23,8 +24,10 @@ struct Launch {
     static Planes<const T> cfl(const void* p, const Geom& g) { return planes_of(static_cast<const T*>(p), Q, g.N); }
     static Planes<T> mfl(void* p, const Geom& g) { return planes_of(static_cast<T*>(p), Q, g.N); }
 
-    // Boxes whose kernels take the EARLY instances (wait_previous): the launch gap counts there.
-    static bool early(const Geom& g) { return g.N <= (1u << 21); }
+    // Boxes whose kernels take the EARLY instances (wait_previous): the launch gap counts there. Not FP64,
+    // whose blocks have to be spread evenly over the FP64 pipes: set up while the previous kernel still
+    // runs they are not (D2Q9 128 x 300 8.5 -> 15.4 us a step, D3Q27 26 x 23 x 31 15.7 -> 31.7).
+    static bool early(const Geom& g) { return S != 1 && g.N <= (1u << 21); }
 #define LBM_UNWRAP(...) __VA_ARGS__
 #define LBM_EARLY(K, PARAMS, GRID, BLOCK, ...)                                                     \
     do {                                                                                           \
@@ -74,14 +77,14 @@ struct Launch {
         return (unsigned)((t + CELLS2_THREADS - 1) / CELLS2_THREADS);
     }
 
-    // FP64 steps are bound by the FP64 pipes, so their blocks have 64 threads: a small box then
-    // reaches every SM (64^2 ran on 16 of them: 11.2 -> 4.6 us a step with the FP64 collision of
-    // bgk_raw; 33 x 29 x 41 37.3 -> 29.5 us against 256 threads; from 64^3 up there is no
-    // difference). A box too tall for 64-thread blocks (grid.y) keeps 256.
+    // FP64 steps are bound by the FP64 pipes, one per scheduler of an SM, so they run single warps as
+    // blocks, which spread evenly: us a step with 32, 64, 128 and 256 threads, D2Q9 64^2 4.4, 4.4, 4.9, 8.2;
+    // 96 x 198 5.2, 5.2, 5.2, 8.6; D3Q19 33 x 29 x 41 29.7, 29.6, 36.4, 37.4; D3Q27 42 x 35 x 22 29.4, 31.2,
+    // 31.4, 41.2; from 64^3 up they are alike. A box too tall for such blocks (grid.y) keeps 256.
     static Shape shape_step(const Geom& g) {
         const int nzp = g.nz - 2 * LBM_SLAB;
         if (S == 1) {
-            const Shape small = shape_for(g, nzp, 64);
+            const Shape small = shape_for(g, nzp, 32);
             if (small.grid.y <= 65535u) return small;
         }
         return shape_for(g, nzp);
@@ -383,13 +386,18 @@ struct Launch {
         }
         return sms;
     }
-    static bool twice(const Geom& g) {
-        if constexpr (TWICE) return !g.link && twice_pays(g, sm_count());
-        return false;
+    // D2Q9 FP32 storage in whole boxes (lbm_plane.cuh)
+    static constexpr bool PLANE = (S == 0 || S == 2) && Q == 9;
+    static int steps_at_once(const Geom& g, long long left) {
+        if (g.link || left < 2) return 1;
+        if constexpr (TWICE) return twice_pays(g, sm_count()) ? 2 : 1;
+        if constexpr (PLANE) return plane_steps(g, sm_count(), left);
+        return 1;
     }
 
-    static cudaError_t step_twice(const Geom& g, const void* coef, const void* src, void* dst, int* flag,
-                                  cudaStream_t st) {
+    static cudaError_t step_several(const Geom& g, const void* coef, int steps, const void* src, void* dst, int* flag,
+                                    cudaStream_t st) {
+        const CF& cf = *static_cast<const CF*>(coef);
         if constexpr (TWICE) {
             long long walks = 0;
             const Tiles t = twice_tiles(g, std::max(1, sm_count()), walks);
@@ -397,9 +405,12 @@ struct Launch {
                                                        twice_smem<Q>());
             if (e != cudaSuccess) return e;
             const long long n = t.chunks ? (long long)t.tiles * t.chunks : ((long long)t.tiles * g.nz + t.run - 1) / t.run;
-            k_step_twice<Q, S><<<(unsigned)n, TWICE_THREADS, twice_smem<Q>(), st>>>(
-                g, *static_cast<const CF*>(coef), t, cpl(src, g), mpl(dst, g), flag);
+            k_step_twice<Q, S><<<(unsigned)n, TWICE_THREADS, twice_smem<Q>(), st>>>(g, cf, t, cpl(src, g), mpl(dst, g),
+                                                                                    flag);
             return cudaGetLastError();
+        }
+        if constexpr (PLANE) {
+            return launch_planes<S>(g, cf, sm_count(), steps, cpl(src, g), mpl(dst, g), flag, st);
         }
         return cudaErrorNotSupported;
     }
@@ -419,7 +430,7 @@ struct Launch {
     static const Ops& ops() {
         static const Ops o = {&init,     &step_pull, &step_aa,   &step_pull_sectors, &step_aa_list, &moments,
                               &totals,   &adj_seed,  &adj_step,  &adj_init,          &link_mask,    &ade_pull,
-                              &ade_aa,   &ade_pull_sectors, &step_aa_even_sectors, &twice, &step_twice};
+                              &ade_aa,   &ade_pull_sectors, &step_aa_even_sectors, &steps_at_once, &step_several};
         return o;
     }
 };

@@ -8,8 +8,8 @@ from gpu_util import gpu_run, oracle_run, perm_lib_to_oracle, rand_theta
 pytestmark = pytest.mark.gpu
 
 
-# FP64 steps run 64-thread blocks (rows of 1, 31, 32, 33, 65 cells: remainders of a warp and of a
-# block; 70,001 rows: more than 64-thread blocks can cover in grid.y). Per step the collision
+# FP64 steps run blocks of one warp (rows of 1, 31, 32, 33, 65 cells: remainders of a warp; 70,001 rows:
+# more than such blocks can cover in grid.y). Per step the collision
 # rounds each population to about 10 * 2^-53 of f <= 0.5, so 20 steps stay below 1e-13.
 @pytest.mark.parametrize("scheme", ["pull", "aa"])
 @pytest.mark.parametrize("q,dims", [(9, (1, 7, 1)), (9, (31, 9, 1)), (9, (65, 4, 1)), (9, (2, 70001, 1)),
@@ -84,3 +84,31 @@ def test_fp16_two_cells_match_one_cell(q, dims, frac):
             assert torch.equal(run("fp16s", scheme, iso, steps), run("fp16w", scheme, iso, steps))
         Th = rand_theta(8, d)
         assert torch.equal(run("fp16s", "pull", Th, steps), run("fp16s", "aa", Th, steps))
+
+
+# D2Q9 FP32 runs eight or four steps per launch on tiles of 8 x 8 to 16 x 16 cells with rings of 3 or 7
+# cells: boxes smaller than the rings, rows and columns left over, one box for each tile size; the
+# step counts leave remainders of 8, 4 and 1, with and without graphs, checks and checkpoints.
+@pytest.mark.parametrize("storage", ["fp32s", "fp32"])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (5, 3, 1), (96, 80, 1), (37, 400, 1), (130, 129, 1), (301, 200, 1)])
+def test_steps_of_a_plane_match_single_steps(dims, storage):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    N = int(np.prod(dims))
+    Th = rand_theta(3, 2)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rho = 1 + 0.02 * torch.randn(N, device="cuda", generator=g)
+    u = 0.03 * torch.randn(2, N, device="cuda", generator=g)
+    runs = []
+    for pieces, kw in (([1] * 53, {}), ([16, 24, 13], {}), ([53], {"use_graphs": -1}), ([53], {"check_every": 11}),
+                       ([7, 46], {"use_graphs": 1})):
+        L = lbm.LBM(9, *dims, 0.62, Th, storage=storage, **kw)
+        L.record_checkpoints(19 if "check_every" in kw else 0)
+        L.init(rho, u)
+        before = L.launches
+        for n in pieces:
+            L.step(n)
+        runs.append((L.launches - before, L.populations(), L.get_state()))
+    assert runs[0][0] == 53 and all(r[0] < 30 for r in runs[1:])
+    for _, f, s in runs:
+        assert torch.equal(f, runs[0][1]) and torch.equal(s, runs[0][2])
