@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S
 // Each thread writes exactly the slots it read, so the in-place update is race free. The link
 // bit of x + c_i is the bit of direction opp(i).
 // ---------------------------------------------------------------------------------------------
-template <int Q, int S, bool MASK, int ODD, bool RAW = false>
+template <int Q, int S, bool MASK, int ODD, bool RAW = false, bool SELECT = true>
 __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<typename Store<S>::T>& cf,
                                          const Planes<typename Store<S>::type>& dst,
                                          const typename Store<S>::T (&d)[Q]) {
@@ -560,7 +560,9 @@ __device__ __forceinline__ void aa_store(const Cell& c, uint32_t lw, const Coef<
             p = dst.p[opp(i)] + c.n;
         } else {
             const Vec3 v = vel<Q>(i);
-            if (MASK) {  // one select of an offset from the lower plane of the pair, as in gather (the odd
+            if (MASK && !SELECT) {
+                p = link_bit(lw, opp(i)) ? dst.p[opp(i)] + c.n : dst.p[i] + off_plus(c, v);
+            } else if (MASK) {  // one select of an offset from the lower plane of the pair, as in gather (the odd
                 // step over the fluid-cell list, porous D3Q27 160^3: 104 -> 94 us)
                 const int lo = i < opp(i) ? i : opp(i);
                 const uint32_t offp = off_plus(c, v) + (i > lo ? c.N : 0u);

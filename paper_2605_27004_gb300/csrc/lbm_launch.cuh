@@ -5,6 +5,7 @@
 #include "lbm_ade.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_adjoint2.cuh"
+#include "lbm_lanes.cuh"
 #include "lbm_pairs.cuh"
 #include "lbm_plane.cuh"
 #include "lbm_quads.cuh"
@@ -90,6 +91,11 @@ struct Launch {
         return shape_for(g, nzp);
     }
 
+    // D2Q9 FP64: four lanes per cell (lbm_lanes.cuh) while every scheduler (four per SM) gets one warp
+    // at most; with two, 80^2 takes the 4.6 us of one lane per cell, and 96 x 80 5.3.
+    static constexpr bool LANES = S == 1 && Q == 9;
+    static bool lanes(const Geom& g) { return !g.link && (g.N + 7) / 8 <= 4u * (uint32_t)sm_count(); }
+
     static cudaError_t step_pull(const Geom& g, const void* coef, const void* src, void* dst, int* flag,
                                  cudaStream_t st) {
         const Shape sh = shape_step(g);
@@ -111,6 +117,13 @@ struct Launch {
             }
             if (odd_rows(g)) {
                 LBM_EARLY(k_step_pull_rows2, (Q), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
+                return cudaGetLastError();
+            }
+        }
+        if constexpr (LANES) {
+            if (lanes(g)) {
+                k_step_lanes<LAYOUT_PULL><<<(g.N + 7) / 8, 32, 0, st>>>(g, cf, static_cast<const double*>(src),
+                                                                       static_cast<double*>(dst), flag);
                 return cudaGetLastError();
             }
         }
@@ -153,6 +166,17 @@ struct Launch {
                     LBM_EARLY(k_step_aa_rows2, (Q, 1), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
                 else
                     LBM_EARLY(k_step_aa_rows2, (Q, 0), blocks_rows2(g), CELLS2_THREADS, g, cf, a, b, flag);
+                return cudaGetLastError();
+            }
+        }
+        if constexpr (LANES) {
+            if (lanes(g)) {
+                const auto from = static_cast<const double*>(src);
+                const auto to = static_cast<double*>(dst);
+                if (odd)
+                    k_step_lanes<LAYOUT_AAODD><<<(g.N + 7) / 8, 32, 0, st>>>(g, cf, from, to, flag);
+                else
+                    k_step_lanes<LAYOUT_LOCAL><<<(g.N + 7) / 8, 32, 0, st>>>(g, cf, from, to, flag);
                 return cudaGetLastError();
             }
         }

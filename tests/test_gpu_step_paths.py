@@ -9,10 +9,11 @@ pytestmark = pytest.mark.gpu
 
 
 # FP64 steps run blocks of one warp (rows of 1, 31, 32, 33, 65 cells: remainders of a warp; 70,001 rows:
-# more than such blocks can cover in grid.y). Per step the collision
+# more than such blocks can cover in grid.y), and D2Q9 boxes of up to 4,864 cells four lanes per cell
+# (7 and 260 cells: a last warp of seven cells and of four; 97 x 51 is past that size). Per step the collision
 # rounds each population to about 10 * 2^-53 of f <= 0.5, so 20 steps stay below 1e-13.
 @pytest.mark.parametrize("scheme", ["pull", "aa"])
-@pytest.mark.parametrize("q,dims", [(9, (1, 7, 1)), (9, (31, 9, 1)), (9, (65, 4, 1)), (9, (2, 70001, 1)),
+@pytest.mark.parametrize("q,dims", [(9, (1, 7, 1)), (9, (31, 9, 1)), (9, (65, 4, 1)), (9, (97, 51, 1)), (9, (2, 70001, 1)),
                                     (19, (33, 3, 5)), (19, (32, 4, 2)), (27, (65, 2, 3))])
 def test_fp64_step_block_edges(q, dims, scheme):
     d, N = (2 if q == 9 else 3), int(np.prod(dims))
