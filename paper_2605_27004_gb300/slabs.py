@@ -236,6 +236,8 @@ class SlabGroup:
         failure (the other threads leave at the broken barrier)."""
         import torch
         errs = [None] * self.nslabs
+        for s in self.streams:  # fields made on the caller's stream are read on the slabs' streams
+            s.wait_stream(torch.cuda.current_stream(self.device))
 
         def work(r):
             try:

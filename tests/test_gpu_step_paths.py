@@ -58,9 +58,9 @@ def test_two_steps_per_launch_match_single_steps(dims, pays, storage):
 # FP16 storage in rows of odd length, and AA with walls: two cells per thread. The FP16 form shifted by
 # the weights runs one cell per thread, and at Theta = cs2 I its stored values and its arithmetic
 # are the same, so the two give the same bits; so do pull and AA, which round the same post-collision
-# values. Rows of 3 to 67 cells (halves of one length and of two), boxes of an odd number of cells and
+# values. Rows of 3 to 387 cells (halves of one length and of two), boxes of an odd number of cells and
 # of a number that is no multiple of a sector's 16, boxes of one row and one plane.
-@pytest.mark.parametrize("q,dims,frac", [(9, (67, 9, 1), 0.0), (9, (3, 1, 1), 0.0), (19, (35, 4, 3), 0.0),
+@pytest.mark.parametrize("q,dims,frac", [(9, (387, 391, 1), 0.0), (9, (67, 9, 1), 0.0), (19, (3, 1, 1), 0.0), (19, (35, 4, 3), 0.0),
                                          (27, (31, 3, 2), 0.0), (19, (5, 1, 7), 0.0), (9, (18, 9, 1), 0.2),
                                          (19, (33, 4, 5), 0.2), (19, (7, 5, 3), 0.3), (27, (6, 5, 3), 0.3),
                                          (27, (40, 6, 5), 0.5), (27, (16, 2, 1), 0.1)])
@@ -113,3 +113,28 @@ def test_steps_of_a_plane_match_single_steps(dims, storage):
     assert runs[0][0] == 53 and all(r[0] < 30 for r in runs[1:])
     for _, f, s in runs:
         assert torch.equal(f, runs[0][1]) and torch.equal(s, runs[0][2])
+
+
+def test_slab_group_waits_for_fields_of_the_callers_stream():
+    """SlabGroup reads the slabs' fields on the slabs' streams: the kernels that cut them out of the box on
+    the caller's stream (held back here by bounded spins of some 10 ms) have to end first."""
+    import torch
+    from paper_2605_27004_gb300 import slabs
+    dims, N = (12, 5, 8), 12 * 5 * 8
+    rho0, u0 = (torch.as_tensor(a, device="cuda") for a in inputs.noise_field(N, 3, 0.05, 3, rho_amp=0.02))
+    got = []
+    for hold in (True, False):
+        G = slabs.SlabGroup(19, *dims, 0.7, rand_theta(1, 3), 4, storage="fp64")
+        if hold:
+            cut = G._slab_fields
+
+            def late(x, r):
+                part = cut(x, r)
+                torch.cuda._sleep(20_000_000)
+                return part * 1.0
+
+            G._slab_fields = late
+        G.init(rho0, u0)
+        G.step(2)
+        got.append(G.populations())
+    assert torch.equal(got[0], got[1])
