@@ -130,10 +130,10 @@ __device__ __forceinline__ typename Store<S>::T from_shifted(typename Store<S>::
 // set up as soon as all of this one's have started, and waits for the previous kernel's writes. They
 // read populations, lambda and velocities with ordinary loads, since a non-coherent load may be moved
 // above the wait, and pointers whose memory another kernel writes are not declared __restrict__.
-// Measured per step: D2Q9 64^2 1.67 -> 1.54 us, D3Q19 64^3 FP32 6.3 -> 5.6 us (graph launches), three
-// launches of a flow coupled to a scalar at 96 x 88 x 80 53 -> 44 us. Above 2M cells the wait at the
-// head of every block costs more than the overlap gives (D3Q27 FP32 256^3 521 -> 542 us, D3Q19 FP16
-// 320^3 441 -> 487 us), so larger boxes keep the plain instances.
+// Measured per step: D3Q19 64^3 FP32 6.3 -> 5.6 us (graph launches), three launches of a flow coupled to a
+// scalar at 96 x 88 x 80 53 -> 44 us. Above 2M cells the wait at the head of every block costs more than
+// the overlap gives (D3Q27 FP32 256^3 521 -> 542 us, D3Q19 FP16 320^3 441 -> 487 us), so larger boxes
+// keep the plain instances.
 template <bool EARLY>
 __device__ __forceinline__ void wait_previous() {
     if constexpr (EARLY) {

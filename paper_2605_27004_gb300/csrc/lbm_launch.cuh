@@ -25,14 +25,24 @@ struct Launch {
     static Planes<const T> cfl(const void* p, const Geom& g) { return planes_of(static_cast<const T*>(p), Q, g.N); }
     static Planes<T> mfl(void* p, const Geom& g) { return planes_of(static_cast<T*>(p), Q, g.N); }
 
-    // Boxes whose kernels take the EARLY instances (wait_previous): the launch gap counts there. Not FP64,
-    // whose blocks have to be spread evenly over the FP64 pipes: set up while the previous kernel still
-    // runs they are not (D2Q9 128 x 300 8.5 -> 15.4 us a step, D3Q27 26 x 23 x 31 15.7 -> 31.7).
-    static bool early(const Geom& g) { return S != 1 && g.N <= (1u << 21); }
+    // Launches that take the EARLY instances (wait_previous): the launch gap counts there. Blocks set up
+    // while the previous kernel still runs are not spread evenly, so not where an SM gets one to three
+    // of them (D3Q19 FP16 64 x 40 x 50, 250 blocks: 3.3 -> 3.6 us a step; D2Q9 301 x 250, 295 blocks: 2.2 ->
+    // 2.5; up to four of the D3Q27 FP16 pair blocks: 64 x 40 x 50 4.0 -> 4.2), nor for FP64, bound by the
+    // FP64 pipes of the SMs (D2Q9 128 x 300 8.5 -> 15.4, D3Q27 26 x 23 x 31 15.7 -> 31.7). Larger boxes
+    // gain nothing: beyond 2M cells, FP16 beyond 90 MB of two arrays (D3Q19 130 x 100 x 100 24.3 -> 24.9),
+    // D3Q27 beyond 60 (FP32 96 x 70 x 60 11.9 -> 12.1).
+    static bool early(const Geom& g, dim3 grid) {
+        const unsigned long long bytes = 2ull * Q * sizeof(ST) * g.N;
+        if (S == 1 || g.N > (1u << 21) || bytes > (Q == 27 ? 60000000ull : S == 3 ? 90000000ull : ~0ull)) return false;
+        const unsigned long long blocks = (unsigned long long)grid.x * grid.y * grid.z, sms = (unsigned)sm_count();
+        return blocks <= sms || blocks >= (Q == 27 && S == 3 ? 4 : 3) * sms;
+    }
 #define LBM_UNWRAP(...) __VA_ARGS__
 #define LBM_EARLY(K, PARAMS, GRID, BLOCK, ...)                                                     \
     do {                                                                                           \
-        if (early(g)) return launch_after(K<LBM_UNWRAP PARAMS, true>, GRID, BLOCK, st, __VA_ARGS__); \
+        if (early(g, GRID))                                                                        \
+            return launch_after(K<LBM_UNWRAP PARAMS, true>, GRID, BLOCK, st, __VA_ARGS__);         \
         K<LBM_UNWRAP PARAMS, false><<<GRID, BLOCK, 0, st>>>(__VA_ARGS__);                          \
     } while (0)
 
@@ -72,7 +82,10 @@ struct Launch {
     static bool quads(const Geom& g) { return S == 3 && Q != 27 && !g.link && (g.nx % 128) == 0; }
 
     // Rows of odd length, FP16 storage without walls: two cells of a row per thread (lbm_cells2.cuh).
-    static bool odd_rows(const Geom& g) { return S == 3 && !g.link && (g.nx % 2) == 1 && g.nx >= 3; }
+    // In small 2D boxes half the threads leave SMs without work (301 x 250 2.2 -> 2.4 us a step).
+    static bool odd_rows(const Geom& g) {
+        return S == 3 && !g.link && (g.nx % 2) == 1 && g.nx >= 3 && (Q != 9 || g.N >= 150000u);
+    }
     static unsigned blocks_rows2(const Geom& g) {
         const unsigned long long t = (unsigned long long)((g.nx + 1) / 2) * g.ny * (g.nz - 2 * LBM_SLAB);
         return (unsigned)((t + CELLS2_THREADS - 1) / CELLS2_THREADS);
