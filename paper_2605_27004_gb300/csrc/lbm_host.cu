@@ -179,6 +179,10 @@ struct lbm_ctx {
     int last_adj_K2 = 0;  // sub-segment length of the last adjoint (== K when flat)
     int last_adj_prefetch = 0;       // host checkpoints the last adjoint restored ahead of use
     std::vector<void*> adj_bufs;     // segment state buffers, kept for later adjoint calls
+    // adj_bufs[1 .. held] hold the states held_t0 + 1 .. held_t0 + held of the current trajectory, left
+    // there by the forward run (step_held)
+    long long held_t0 = -1;
+    int held = 0;
     double grad_theta[6] = {0};
     double grad_tau = 0.0;
 
@@ -419,6 +423,33 @@ cudaError_t launch_steps(lbm_ctx* c, cudaStream_t s, long long left, int* taken)
     c->steps += *taken;
     c->launches += 1;
     return e;
+}
+
+// The last `len` steps of a recorded forward run, from the checkpoint the context is at: every step writes
+// its state into the segment buffer where lbm_adjoint looks for it, instead of the other array (no
+// extra traffic: a step reads one array and writes another), and the last one into the context's.
+// The adjoint then starts without recomputing that segment. The buffers are those an earlier
+// lbm_adjoint allocated. Training steps, K = 20: 128^3 FP32 n = 100
+// 18.1 -> 17.3 ms, 192^3 FP16 AA n = 40 18.9 -> 16.8 ms.
+int step_held(lbm_ctx* c, int len) {
+    const long long t0 = c->steps;
+    const void* src = state_ptr(c);
+    void* last = c->scheme == LBM_PULL2 ? c->pop[c->cur ^ 1] : c->pop[0];
+    for (int j = 0; j < len; ++j) {
+        void* dst = j + 1 < len ? c->adj_bufs[(size_t)j + 1] : last;
+        const cudaError_t e = step_kernel(c, src, dst, t0 + j, c->stream);
+        if (e != cudaSuccess) {
+            c->state_valid = false;
+            return cuda_fail(c, e, "stream-collide kernel");
+        }
+        src = dst;
+        c->launches += 1;
+    }
+    if (c->scheme == LBM_PULL2) c->cur ^= 1;
+    c->steps = t0 + len;
+    c->held_t0 = t0;
+    c->held = len - 1;
+    return LBM_OK;
 }
 
 int ensure_graph(lbm_ctx* c, int gsteps) {
@@ -901,6 +932,7 @@ int lbm_set_params(lbm_ctx* c, double tau, const double* Theta) {
     c->init_fields = false;
     c->grads_ready = false;
     c->rec_valid = 0;
+    c->held = 0;
     return LBM_OK;
 }
 
@@ -928,6 +960,7 @@ int lbm_init(lbm_ctx* c, const void* rho, const void* u) {
     c->init_fields = true;
     c->grads_ready = false;
     c->rec_valid = 0;
+    c->held = 0;
     return record_ckpt(c);
 }
 
@@ -936,6 +969,7 @@ int lbm_record_checkpoints(lbm_ctx* c, int checkpoint_every) {
     if (int rc = flow_only(c, "lbm_record_checkpoints")) return rc;
     c->rec_K = checkpoint_every;
     c->rec_valid = 0;
+    c->held = 0;
     if (checkpoint_every > 0 && c->state_valid && c->steps == 0 && c->init_fields) return record_ckpt(c);
     return LBM_OK;
 }
@@ -948,12 +982,26 @@ int lbm_step(lbm_ctx* c, int n) {
     long long next_check = c->opt.check_every > 0 ? (c->steps / c->opt.check_every + 1) * c->opt.check_every : -1;
     const bool recording = c->rec_K > 0 && c->rec_valid * c->rec_K > c->steps;
     long long next_rec = recording ? (c->steps / c->rec_K + 1) * c->rec_K : -1;
+    // the last segment's states stay in the adjoint's buffers where an earlier adjoint allocated them
+    long long hold_from = -1;
+    if (n > 0) c->held = 0;
+    if (recording && n > 0 && next_check < 0 && !c->slab && c->init_fields) {
+        const long long end = c->steps + n, t0 = (end - 1) / c->rec_K * c->rec_K;
+        if (t0 >= c->steps && end - t0 >= 2 && (long long)c->adj_bufs.size() >= end - t0) {
+            hold_from = t0;
+            graphs = graphs && t0 - c->steps >= gsteps;
+        }
+    }
     int left = n;
     while (left > 0) {
+        if (c->steps == hold_from) {
+            if (int rc = step_held(c, left)) return rc;
+            return next_rec >= 0 && c->steps >= next_rec ? record_ckpt(c) : LBM_OK;
+        }
         const bool aligned = (c->steps & 1) == 0 && (c->scheme != LBM_PULL2 || c->cur == 0);
         bool ran = false;
         if (graphs && left >= gsteps && aligned && (next_check < 0 || c->steps + gsteps <= next_check) &&
-            (next_rec < 0 || c->steps + gsteps <= next_rec)) {
+            (next_rec < 0 || c->steps + gsteps <= next_rec) && (hold_from < 0 || c->steps + gsteps <= hold_from)) {
             int rc = ensure_graph(c, gsteps);
             if (rc) return rc;
             LBM_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
@@ -1095,6 +1143,10 @@ int lbm_adjoint(lbm_ctx* c, const void* loss_grad, int n, int K) {
         }
     }
     const bool flat_plan = W >= K - 1;
+    // the last segment's states are there from the forward run
+    const bool use_held = recorded && flat_plan && c->held > 0 && c->held_t0 == (long long)(C - 1) * K &&
+                          c->held == n - (int)c->held_t0 - 1;
+    c->held = 0;  // this call overwrites them
     const int nbuf = std::max(2, W + 1);
     int longest = K;  // longest sub-segment of a full segment, reported by lbm_adjoint_info
     if (!flat_plan) {
@@ -1321,7 +1373,11 @@ int lbm_adjoint(lbm_ctx* c, const void* loss_grad, int n, int K) {
             }
         }
         if (cs && s > 0 && ckpt_host[s - 1]) LBM_ADJ_CHECK(prefetch(s - 1), "checkpoint prefetch");
-        if (seg_graphs && len == K) {
+        if (use_held && s == C - 1) {
+            std::vector<const void*> st(bufs, bufs + len);
+            st[0] = start;
+            LBM_ADJ_RC(sweep(st, t0));
+        } else if (seg_graphs && len == K) {
             if (start != bufs[0])
                 LBM_ADJ_CHECK(cudaMemcpyAsync(bufs[0], start, SB, cudaMemcpyDeviceToDevice, c->stream),
                               "segment start copy");
@@ -1419,6 +1475,7 @@ int lbm_adjoint_release(lbm_ctx* c) {
     const size_t SB = c->state_bytes(), LB = (size_t)c->q * c->N * c->felem;
     for (void* p : c->adj_bufs) dev_free(c, p, SB);
     c->adj_bufs.clear();
+    c->held = 0;
     dev_free(c, c->lam[0], LB);
     dev_free(c, c->lam[1], LB);
     c->lam[0] = c->lam[1] = nullptr;
@@ -1496,6 +1553,7 @@ int lbm_set_state(lbm_ctx* c, const void* src, size_t bytes) {
     c->init_fields = false;  // the adjoint needs the initial fields of an lbm_init
     c->grads_ready = false;
     c->rec_valid = 0;
+    c->held = 0;
     return LBM_OK;
 }
 

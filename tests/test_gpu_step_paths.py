@@ -138,3 +138,44 @@ def test_slab_group_waits_for_fields_of_the_callers_stream():
         G.step(2)
         got.append(G.populations())
     assert torch.equal(got[0], got[1])
+
+
+# From the second gradient on, the forward run leaves its last segment's states in the adjoint's
+# buffers: the same states as recomputed ones, so the same bits as the first gradient. Whole and cut last
+# segments, one of a single step, a run shorter than a segment; both schemes and parities; in between
+# a run in two pieces (no segment can be held), a second adjoint of the same run, released buffers.
+@pytest.mark.parametrize("n,K", [(24, 6), (23, 5), (21, 5), (9, 20), (22, 7)])
+@pytest.mark.parametrize("storage,scheme", [("fp32s", "pull"), ("fp16s", "aa"), ("fp64", "aa")])
+@pytest.mark.parametrize("graphs", [-1, 1])
+def test_gradient_with_held_segment(n, K, storage, scheme, graphs):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    dims = (18, 7, 6)
+    N = int(np.prod(dims))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    u = (0.03 * torch.randn(3, N, device="cuda", generator=g)).double()
+    w = torch.randn(3, N, device="cuda", generator=g).double()
+    L = lbm.LBM(19, *dims, 0.7, rand_theta(2, 3), storage=storage, scheme=scheme, use_graphs=graphs)
+    L.record_checkpoints(K)
+
+    def gradient(pieces, times=1):
+        L.init(None, u)
+        for m in pieces:
+            L.step(m)
+        f = L.populations()
+        for _ in range(times):
+            before = L.launches
+            L.adjoint(w, n, K)
+            count = L.launches - before
+        dth, dtau, du0 = L.gradients()
+        return f, dth, dtau, du0, count
+
+    first = gradient([n])
+    for pieces, times, release in (([n], 1, False), ([n - 2, 2], 1, False), ([n], 2, False), ([n], 1, True), ([n], 1, False)):
+        if release:
+            L.adjoint_release()
+        again = gradient(pieces, times)
+        assert torch.equal(again[0], first[0]) and torch.equal(again[3], first[3])
+        assert np.array_equal(again[1], first[1]) and again[2] == first[2]
+    held = n - (n - 1) // K * K - 1 if n >= K else 0  # a run shorter than a segment is run again
+    assert again[4] == first[4] - held
