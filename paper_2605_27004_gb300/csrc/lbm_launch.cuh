@@ -91,17 +91,23 @@ struct Launch {
         return (unsigned)((t + CELLS2_THREADS - 1) / CELLS2_THREADS);
     }
 
+    // Block of the list kernels, as in shape_step: porous D3Q27 256^3 FP32 509 -> 499 us a step, FP16 AA 351 ->
+    // 346, 160^3 FP16 pull 103 -> 99.
+    static constexpr unsigned LIST_THREADS = 128;
+    // Block of a one-cell step. 128 threads even out the blocks of an SM sooner than 256: us a step, D3Q19
+    // FP32 AA 64^3 6.3 -> 6.1, 96 x 88 x 80 13.5 -> 12.9, 384^3 1368 -> 1350; D3Q27 FP32 75^3 15.4 -> 14.4,
+    // porous AA 160^3 148 -> 142, scalar 64 x 70 x 60 7.5 -> 7.1. D3Q27 boxes without walls beyond 2M cells are
+    // as fast or 1 % faster with 256 outside the flow's AA steps (pull 256^3 522 against 527).
     // FP64 steps are bound by the FP64 pipes, one per scheduler of an SM, so they run single warps as
     // blocks, which spread evenly: us a step with 32, 64, 128 and 256 threads, D2Q9 64^2 4.4, 4.4, 4.9, 8.2;
     // 96 x 198 5.2, 5.2, 5.2, 8.6; D3Q19 33 x 29 x 41 29.7, 29.6, 36.4, 37.4; D3Q27 42 x 35 x 22 29.4, 31.2,
-    // 31.4, 41.2; from 64^3 up they are alike. A box too tall for such blocks (grid.y) keeps 256.
-    static Shape shape_step(const Geom& g) {
+    // 31.4, 41.2; from 64^3 up they are alike.
+    // A box too tall for such blocks (grid.y) keeps 256.
+    static Shape shape_step(const Geom& g, bool flow_aa = false) {
         const int nzp = g.nz - 2 * LBM_SLAB;
-        if (S == 1) {
-            const Shape small = shape_for(g, nzp, 32);
-            if (small.grid.y <= 65535u) return small;
-        }
-        return shape_for(g, nzp);
+        const bool wide = Q == 27 && !g.link && g.N > (1u << 21) && !flow_aa;
+        const Shape sh = shape_for(g, nzp, S == 1 ? 32 : wide ? 256 : 128);
+        return sh.grid.y <= 65535u ? sh : shape_for(g, nzp);
     }
 
     // D2Q9 FP64: four lanes per cell (lbm_lanes.cuh) while every scheduler (four per SM) gets one warp
@@ -149,7 +155,7 @@ struct Launch {
 
     static cudaError_t step_aa(const Geom& g, const void* coef, int odd, const void* src, void* dst, int* flag,
                                cudaStream_t st) {
-        const Shape sh = shape_step(g);
+        const Shape sh = shape_step(g, true);
         const CF& cf = *static_cast<const CF*>(coef);
         const auto a = cpl(src, g);
         const auto b = mpl(dst, g);
@@ -212,7 +218,8 @@ struct Launch {
         if (L.count == 0) return cudaSuccess;
         const CF& cf = *static_cast<const CF*>(coef);
         const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
-        k_step_pull_sectors<Q, S><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g),
+        k_step_pull_sectors<Q, S><<<(unsigned)((threads + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0,
+                    st>>>(g, cf, L, cpl(src, g), mpl(dst, g),
                                                                                     flag);
         return cudaGetLastError();
     }
@@ -221,11 +228,11 @@ struct Launch {
                                     void* dst, int* flag, cudaStream_t st) {
         if (L.count == 0) return cudaSuccess;
         const CF& cf = *static_cast<const CF*>(coef);
-        const unsigned nb = (L.count + 255) / 256;
+        const unsigned nb = (L.count + LIST_THREADS - 1) / LIST_THREADS;
         if (odd)
-            k_step_aa_list<Q, S, 1><<<nb, 256, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
+            k_step_aa_list<Q, S, 1><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
         else
-            k_step_aa_list<Q, S, 0><<<nb, 256, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
+            k_step_aa_list<Q, S, 0><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
         return cudaGetLastError();
     }
 
@@ -334,7 +341,7 @@ struct Launch {
 
     static cudaError_t ade_pull(const Geom& g, const void* coef, const void* u, const void* src, void* dst, int* flag,
                                 cudaStream_t st) {
-        const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
+        const Shape sh = shape_step(g);
         const CF& cf = *static_cast<const CF*>(coef);
         if constexpr (S == 3) {  // pairs(g) holds for FP16 r-shifted storage only
             if constexpr (Q != 27) {
@@ -363,7 +370,7 @@ struct Launch {
 
     static cudaError_t ade_aa(const Geom& g, const void* coef, const void* u, int odd, const void* src, void* dst,
                               int* flag, cudaStream_t st) {
-        const Shape sh = shape_for(g, g.nz - 2 * LBM_SLAB);
+        const Shape sh = shape_step(g);
         const CF& cf = *static_cast<const CF*>(coef);
         const auto v = vel_field(u, g);
         const auto a = cpl(src, g);
@@ -407,7 +414,8 @@ struct Launch {
         if (L.count == 0) return cudaSuccess;
         const CF& cf = *static_cast<const CF*>(coef);
         const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
-        k_ade_pull_sectors<Q, S><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(g, cf, L, vel_field(u, g),
+        k_ade_pull_sectors<Q, S><<<(unsigned)((threads + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0, st>>>(g,
+                    cf, L, vel_field(u, g),
                                                                                    cpl(src, g), mpl(dst, g), flag);
         return cudaGetLastError();
     }
