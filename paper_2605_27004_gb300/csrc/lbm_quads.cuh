@@ -93,6 +93,36 @@ __device__ __forceinline__ void st_word4(__half* p, F2 a, F2 b) {
     *reinterpret_cast<uint2*>(p) = make_uint2(f2_to_half2_bits(a), f2_to_half2_bits(b));
 }
 
+// The stores of a word of an x-shifted plane in the odd AA step, predicated instead of branched (the
+// warp's end lanes store other parts than the inner ones): `whole` lanes store the word (w0, w1); the
+// others what is theirs of it.
+// c_x = +1: the halves 1 (h) and 2, 3 (w1); with `past`, half `ph` goes to the next warp's word at q.
+__device__ __forceinline__ void st_word4_up(__half* p, unsigned w0, unsigned w1, unsigned short h, bool whole, __half* q,
+                                            unsigned short ph, bool past) {
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\t"
+        "setp.ne.u32 a, %6, 0;\n\tsetp.ne.u32 b, %7, 0;\n\t"
+        "@a st.global.v2.b32 [%0], {%1, %2};\n\t"
+        "@!a st.global.b16 [%0 + 2], %3;\n\t"
+        "@!a st.global.b32 [%0 + 4], %2;\n\t"
+        "@b st.global.b16 [%4], %5;\n\t}"
+        ::"l"(p), "r"(w0), "r"(w1), "h"(h), "l"(q), "h"(ph), "r"((unsigned)whole), "r"((unsigned)past)
+        : "memory");
+}
+// c_x = -1: the halves 0, 1 (w0) and 2 (h); with `past`, half `ph` goes to the previous warp's word at q.
+__device__ __forceinline__ void st_word4_down(__half* p, unsigned w0, unsigned w1, unsigned short h, bool whole, __half* q,
+                                              unsigned short ph, bool past) {
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\t"
+        "setp.ne.u32 a, %6, 0;\n\tsetp.ne.u32 b, %7, 0;\n\t"
+        "@a st.global.v2.b32 [%0], {%1, %2};\n\t"
+        "@!a st.global.b32 [%0], %1;\n\t"
+        "@!a st.global.b16 [%0 + 4], %3;\n\t"
+        "@b st.global.b16 [%4], %5;\n\t}"
+        ::"l"(p), "r"(w0), "r"(w1), "h"(h), "l"(q), "h"(ph), "r"((unsigned)whole), "r"((unsigned)past)
+        : "memory");
+}
+
 // ---------------------------------------------------------------------------------------------
 // Pull step, four cells per thread (FP16 r-shifted storage: the stored value is d = f - r).
 // ---------------------------------------------------------------------------------------------
@@ -167,10 +197,13 @@ __global__ void __launch_bounds__(256, 2)
     // row start or the successor of another warp's lane 31. For c_x = +-1 the value that belongs to
     // the thread's own aligned word but comes from the neighbouring lane's cell is taken by a warp
     // shuffle, and the word is stored whole; only the warp's end lanes store single halves across
-    // the warp boundary. Each slot is still written after the lane that gathered it has gathered it:
-    // the shuffled value depends on that lane's gather (measured for the flow at 256^3 / 512^3 /
-    // 768^3: AA 0.843 -> 0.854 / 0.864 -> 0.888 / 0.874 -> 0.867).
+    // the warp boundary, predicated: as branches the ten planes cost 0.7 stalls an instruction in
+    // branch resolving (D3Q19 256^3 / 512^3 / 128^3 222 / 1716 / 25.2 -> 211 / 1641 / 23.5 us a step of the AA
+    // pair; the scalar, which had kept three stores a plane, 257 -> 252 at 256^3, D2Q9 1024^2 9.1 -> 8.0).
+    // Each slot is still written after the lane that gathered it has gathered it: the shuffled value
+    // depends on that lane's gather.
     const int lane = (threadIdx.x + threadIdx.y * blockDim.x) & 31;
+    const int xn = c.x0 + 4 == nx ? 0 : c.x0 + 4, xp = c.x0 == 0 ? nx - 1 : c.x0 - 1;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const Vec3 v = vel<Q>(i);
@@ -180,33 +213,14 @@ __global__ void __launch_bounds__(256, 2)
             continue;
         }
         const unsigned wa = f2_to_half2_bits(da[i]), wb = f2_to_half2_bits(db[i]);
-        if constexpr (ADE) {  // the scalar keeps the three stores per plane (measured 0.851 -> 0.833 with shuffles)
-            const int xf = v.x == 1 ? c.x0 + 1 : (c.x0 == 0 ? nx - 1 : c.x0 - 1);
-            const int xm = v.x == 1 ? c.x0 + 2 : c.x0;
-            const int xl = v.x == 1 ? (c.x0 + 4 == nx ? 0 : c.x0 + 4) : c.x0 + 2;
-            *reinterpret_cast<unsigned short*>(row + xf) = (unsigned short)(wa & 0xffffu);
-            *reinterpret_cast<unsigned*>(row + xm) = mid_halves(wa, wb);
-            *reinterpret_cast<unsigned short*>(row + xl) = (unsigned short)(wb >> 16);
-        } else if (v.x == 1) {  // targets x0 + 1 .. x0 + 4: own word gets (lane - 1's last, a.x, a.y, b.x)
+        if (v.x == 1) {  // targets x0 + 1 .. x0 + 4: own word gets (lane - 1's last, a.x, a.y, b.x)
             const unsigned prev = __shfl_up_sync(0xffffffffu, wb >> 16, 1);
-            if (lane != 0) {
-                *reinterpret_cast<uint2*>(row + c.x0) = make_uint2((prev & 0xffffu) | (wa << 16), mid_halves(wa, wb));
-            } else {
-                *reinterpret_cast<unsigned short*>(row + c.x0 + 1) = (unsigned short)(wa & 0xffffu);
-                *reinterpret_cast<unsigned*>(row + c.x0 + 2) = mid_halves(wa, wb);
-            }
-            if (lane == 31)  // into the next warp's word (or the row start)
-                *reinterpret_cast<unsigned short*>(row + (c.x0 + 4 == nx ? 0 : c.x0 + 4)) = (unsigned short)(wb >> 16);
+            st_word4_up(row + c.x0, (prev & 0xffffu) | (wa << 16), mid_halves(wa, wb), (unsigned short)(wa & 0xffffu),
+                        lane != 0, row + xn, (unsigned short)(wb >> 16), lane == 31);
         } else {  // targets x0 - 1 .. x0 + 2: own word gets (a.y, b.x, b.y, lane + 1's first)
             const unsigned next = __shfl_down_sync(0xffffffffu, wa & 0xffffu, 1);
-            if (lane != 31) {
-                *reinterpret_cast<uint2*>(row + c.x0) = make_uint2(mid_halves(wa, wb), (wb >> 16) | (next << 16));
-            } else {
-                *reinterpret_cast<unsigned*>(row + c.x0) = mid_halves(wa, wb);
-                *reinterpret_cast<unsigned short*>(row + c.x0 + 2) = (unsigned short)(wb >> 16);
-            }
-            if (lane == 0)  // into the previous warp's word (or the row end)
-                *reinterpret_cast<unsigned short*>(row + (c.x0 == 0 ? nx - 1 : c.x0 - 1)) = (unsigned short)(wa & 0xffffu);
+            st_word4_down(row + c.x0, mid_halves(wa, wb), (wb >> 16) | (next << 16), (unsigned short)(wb >> 16),
+                          lane != 31, row + xp, (unsigned short)(wa & 0xffffu), lane == 0);
         }
     }
 }
