@@ -128,7 +128,9 @@ int lbm_set_params(lbm_ctx* ctx, double tau, const double* Theta);
  * cells are ignored. Resets the step counter; the fields are kept for lbm_adjoint. */
 int lbm_init(lbm_ctx* ctx, const void* rho, const void* u);
 
-/* Advance n >= 0 time steps of Eq. LBE_BGK: one fused stream + collide kernel per step. */
+/* Advance n >= 0 time steps of Eq. LBE_BGK: fused stream + collide kernels of one step, or of several
+ * where FP32 pull boxes without walls allow it (D3Q19 two, D2Q9 four or eight steps per launch, with the
+ * bits of single steps; stops for check_every and recorded checkpoints are kept). */
 int lbm_step(lbm_ctx* ctx, int n);
 
 /* Macroscopic fields of f(t): rho = sum f_i, u = sum f_i c_i / rho (Eqs. a0discrete_f,
@@ -162,7 +164,9 @@ int lbm_record_checkpoints(lbm_ctx* ctx, int checkpoint_every);
  * copied back on a second stream one segment ahead of use when one more state fits on the
  * device. Leaves f(n) in place. Results are read with lbm_gradients. The working set (two lambda
  * arrays, the segment states) is allocated by the first call and kept for later calls (an
- * optimisation loop pays for it once) until lbm_adjoint_release or lbm_destroy. Synchronises. */
+ * optimisation loop pays for it once) until lbm_adjoint_release or lbm_destroy. From then on the last
+ * lbm_step of a recorded run leaves the states of its last segment in that working set, and the
+ * adjoint does not recompute them. Synchronises. */
 int lbm_adjoint(lbm_ctx* ctx, const void* loss_grad, int n, int checkpoint_every);
 
 /* Plan of the last lbm_adjoint: sub_segment = the longest sub-segment of a full segment when

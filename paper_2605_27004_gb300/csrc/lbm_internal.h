@@ -22,13 +22,13 @@ struct Geom {
 constexpr uint32_t LINK_SOLID = 0x80000000u;
 
 // The fluid cells of a box with walls, listed in increasing cell index, so that a kernel can give
-// every lane of a warp a fluid cell (FP16 AA steps); or, for the FP16 pull step, the 16-cell
-// groups (one 32-byte sector of every FP16 plane) that hold at least one fluid cell (rows of the porous medium are about 30 % solid, and a lane
-// of a solid cell still issues every instruction of its warp). A cell's coordinates come back
-// from its index by exact reciprocal multiplication: n / d = umul64hi(n, ceil(2^64 / d)) for
-// n, d < 2^32 and d >= 2. The link words stand beside the list, so that a lane fetches them together
-// with its entry and not after it (porous D3Q27 256^3,
-// FP16: pull 450 -> 429, AA 361 -> 349 us a step).
+// every lane of a warp a fluid cell (FP16 AA steps); or, for the pull steps, the groups of 16 FP16 or 8
+// FP32 cells (one 32-byte sector of a plane) that hold at least one fluid cell (rows of the porous
+// medium are about 30 % solid, and a lane of a solid cell still issues every instruction of its
+// warp). A cell's coordinates come back from its index by exact reciprocal multiplication:
+// n / d = umul64hi(n, ceil(2^64 / d)) for n, d < 2^32 and d >= 2. The link words stand beside the list, so
+// that a lane fetches them together with its entry and not after it (porous D3Q27 256^3, FP16: pull
+// 450 -> 429, AA 361 -> 349 us a step).
 struct CellList {
     const uint32_t* idx;
     const uint32_t* link;  // the link words of the listed cells (all cells of a listed sector), in list order
@@ -67,7 +67,8 @@ struct Coef {
 //   AAODD  f_i(x) = A[opp i][x - c_i], or A[i][x] if x - c_i is solid (AA, odd step count)
 enum Layout { LAYOUT_LOCAL = 0, LAYOUT_PULL = 1, LAYOUT_AAODD = 2 };
 
-// Launch shape shared by every per-cell kernel: 256-thread blocks, x fastest, one grid plane per
+// Launch shape of the per-cell kernels: blocks of `threads` (256 unless a kernel's rule says less; the
+// gradient and totals records are one per 256-thread block), x fastest, one grid plane per
 // processed lattice plane (nzp of them).
 struct Shape {
     dim3 grid, block;

@@ -504,7 +504,8 @@ __device__ __forceinline__ bool store_group(unsigned act, bool solid) {
 
 // ---------------------------------------------------------------------------------------------
 // Fused stream + collide, two arrays, pull form: gather f(t) from the post-collision array of
-// the previous step, relax, store at the own cell. One launch per time step.
+// the previous step, relax, store at the own cell. One launch per time step (several steps per launch:
+// lbm_twice.cuh, lbm_plane.cuh).
 // ---------------------------------------------------------------------------------------------
 template <int Q, int S, bool MASK, bool EARLY>
 __global__ void __launch_bounds__(256) k_step_pull(Geom g, Coef<typename Store<S>::T> cf,

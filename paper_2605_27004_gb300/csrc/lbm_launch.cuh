@@ -92,8 +92,12 @@ struct Launch {
     }
 
     // Block of the list kernels, as in shape_step: porous D3Q27 256^3 FP32 509 -> 499 us a step, FP16 AA 351 ->
-    // 346, 160^3 FP16 pull 103 -> 99.
+    // 346, 160^3 FP16 pull 103 -> 99; only the D3Q27 FP16 pull step of large boxes is faster with 256 (256^3
+    // 432 against 451).
     static constexpr unsigned LIST_THREADS = 128;
+    static unsigned pull_list_threads(unsigned long long cells) {
+        return Q == 27 && sizeof(ST) == 2 && cells > 8000000ull ? 256u : LIST_THREADS;
+    }
     // Block of a one-cell step. 128 threads even out the blocks of an SM sooner than 256: us a step, D3Q19
     // FP32 AA 64^3 6.3 -> 6.1, 96 x 88 x 80 13.5 -> 12.9, 384^3 1368 -> 1350; D3Q27 FP32 75^3 15.4 -> 14.4,
     // porous AA 160^3 148 -> 142, scalar 64 x 70 x 60 7.5 -> 7.1. D3Q27 boxes without walls beyond 2M cells are
@@ -218,9 +222,9 @@ struct Launch {
         if (L.count == 0) return cudaSuccess;
         const CF& cf = *static_cast<const CF*>(coef);
         const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
-        k_step_pull_sectors<Q, S><<<(unsigned)((threads + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0,
-                    st>>>(g, cf, L, cpl(src, g), mpl(dst, g),
-                                                                                    flag);
+        const unsigned bt = pull_list_threads(threads);
+        k_step_pull_sectors<Q, S><<<(unsigned)((threads + bt - 1) / bt), bt, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g),
+                                                                                      flag);
         return cudaGetLastError();
     }
 
