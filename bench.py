@@ -44,7 +44,7 @@ ELEM = {"fp32": 4, "fp32s": 4, "fp16s": 2, "fp16w": 2, "fp64": 8}
 # kernel change the bench reports traffic = null (with the reason) until the capture is redone.
 NCU_TRAFFIC = {
     # mean of 3 launches at 256^3: read 1.27521e9 + write 1.22052e9 bytes
-    "d3q19_fp32s_pull": {"traffic_bytes": 2.4957e+09, "kernel_sha": "d1d5effa5735a487"},
+    "d3q19_fp32s_pull": {"traffic_bytes": 2.4954e+09, "kernel_sha": "47e8ec1cd73c9c0e"},
 }
 
 
@@ -613,7 +613,8 @@ def run_profile(args, torch, lbm):
     kind = ("ade_porous" if args.ade else "porous") if args.porous else "ade" if args.ade else "tg"
     L, _ = make_ctx(args.lattice, args.n, args.storage, args.scheme, kind, torch, lbm, use_graphs=-1)
     if args.kernel == "fwd":
-        L.step(args.warmup + args.steps)
+        for _ in range(args.warmup + args.steps):  # one launch each
+            L.step(1)
     else:
         L.step(args.steps)
         g = torch.randn(L.d, L.N, device="cuda", dtype=torch.float64 if args.storage == "fp64" else torch.float32)
