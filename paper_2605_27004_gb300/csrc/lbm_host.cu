@@ -1329,8 +1329,14 @@ int lbm_adjoint(lbm_ctx* c, const void* loss_grad, int n, int K) {
     // not a restore target), and no halo callbacks between the kernels.
     int n_host_ckpt = 0;
     for (int k = 0; k < C; ++k) n_host_ckpt += ckpt_host[k] ? 1 : 0;
+    // From half a million cells on, FP32 kernels outlast their launches, and without a graph the
+    // segment's start is read where it lies instead of copied. One step (recompute and adjoint, K =
+    // 20) in us, with and without graphs: D3Q19 pull 80^3 39.5 / 38.3, 128^3 131.9 / 129.6; D3Q19 AA
+    // 96^3 63.6 / 61.8; D2Q9 720^2 23.8 / 21.9, 1024^2 42.2 / 40.5. D3Q27 and FP16 keep the graphs:
+    // D3Q27 96^3 107.4 / 109.5, D3Q19 FP16 112^3 76.4 / 78.9.
+    const long long graph_cells = c->elem == 4 && c->q != 27 ? 500000 : 1LL << 21;
     const bool seg_graphs = flat_plan && K % 2 == 0 && K >= 2 && n_host_ckpt == 0 && !c->slab &&
-                            (c->opt.use_graphs > 0 || (c->opt.use_graphs == 0 && c->N <= (1LL << 21)));
+                            (c->opt.use_graphs > 0 || (c->opt.use_graphs == 0 && c->N <= graph_cells));
     auto capture_segment = [&](long long t0) -> int {
         if (!c->cap_stream) LBM_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
         LBM_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
