@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(32)
     double h = LAYOUT == LAYOUT_PULL ? src[pg + plus] : LAYOUT == LAYOUT_LOCAL ? src[pg + n] : src[pf + plus];
     double rho, usum;
     bgk_lane(cf, j, rest, f, h, rho, usum);
+    __syncwarp();  // in place, lane 0 writes the rest population that the cell's other lanes have read
     if (!in) return;
     if (!(rho > 0.0) || !isfinite(usum)) *flag = 1;
     if (j == 0) dst[n] = rest;

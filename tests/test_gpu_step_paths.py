@@ -24,6 +24,18 @@ def test_fp64_step_block_edges(q, dims, scheme):
     assert np.abs(g["f"] - o["f"][:, perm_lib_to_oracle(q)].T).max() < 1e-13
 
 
+# Four lanes per cell read a cell's rest population and one of them replaces it, in place in the AA
+# pattern: the values that are rounded are those of the pull scheme, so the bits are the same. Boxes of
+# one warp, of a last warp with spare lanes, and of the largest size that runs so.
+@pytest.mark.parametrize("dims", [(3, 2, 1), (33, 7, 1), (64, 64, 1), (76, 64, 1)])
+def test_fp64_lanes_in_place_match_pull(dims):
+    Th = rand_theta(5, 2)
+    rho0, u0 = inputs.noise_field(int(np.prod(dims)), 2, 0.05, 6, rho_amp=0.02)
+    for steps in (200, 201):
+        f = [gpu_run(9, dims, 0.8, Th, rho0, u0, steps, storage="fp64", scheme=s)["f"] for s in ("pull", "aa")]
+        assert np.array_equal(f[0], f[1])
+
+
 # D3Q19 FP32 boxes run two steps per launch: the same arithmetic, so the same bits as single steps.
 # Tiles of 64 x 9 cells: rows in one, two and three tiles (the last narrower), rows left over in y,
 # planes split among blocks in chunks of one tile and in runs over several; odd step counts, and
