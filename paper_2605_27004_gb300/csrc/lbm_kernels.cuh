@@ -1129,8 +1129,9 @@ __global__ void __launch_bounds__(256, S == 1 ? 1 : Q == 27 ? 2 : 4) k_adj_step(
     using T = typename Store<S>::T;
     T rec[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
     Cell c;
-    if (make_cell(g, c)) {
-        wait_previous<EARLY>();
+    const bool in = make_cell(g, c);
+    wait_previous<EARLY>();  // threads outside the box too: they add to the block's record
+    if (in) {
         const uint32_t lw = link_of<MASK>(g, c);
         if (!(MASK && (lw & LINK_SOLID))) {
             // mu = S^T lambda_{t+1}: reverse gather along +c_i

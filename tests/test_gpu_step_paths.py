@@ -191,3 +191,40 @@ def test_gradient_with_held_segment(n, K, storage, scheme, graphs):
         assert np.array_equal(again[1], first[1]) and again[2] == first[2]
     held = n - (n - 1) // K * K - 1 if n >= K else 0  # a run shorter than a segment is run again
     assert again[4] == first[4] - held
+
+
+# The adjoint's steps add to the gradient records of the step before, and are set up while that one
+# runs: their sums against those of a process that waits for every launch, bit for bit. Rows that leave
+# fewer than the eight threads of a record in the last block of a row (5, 260 and 33 cells).
+def _gradients_of_short_rows(path):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    out = []
+    for q, dims in ((19, (5, 6, 4)), (19, (260, 3, 2)), (9, (33, 5, 1))):
+        d, N = (2 if q == 9 else 3), int(np.prod(dims))
+        rho0, u0 = inputs.noise_field(N, d, 0.05, 6, rho_amp=0.02)
+        w = np.random.default_rng(4).standard_normal((d, N))
+        for scheme in ("pull", "aa"):
+            L = lbm.LBM(q, *dims, 0.7, rand_theta(2, d), scheme=scheme, use_graphs=-1)
+            L.init(torch.as_tensor(rho0), torch.as_tensor(u0))
+            L.step(40)
+            L.adjoint(torch.as_tensor(w), 40, 20)
+            dth, dtau, du0 = L.gradients()
+            out.append(np.concatenate([dth, [dtau], du0.double().cpu().numpy().ravel()]))
+    np.save(path, np.concatenate(out))
+
+
+def test_gradient_records_match_waited_launches(tmp_path):
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    got = []
+    for wait in ("0", "1"):
+        path = str(tmp_path / f"{wait}.npy")
+        code = (f"import sys; sys.path[:0] = [{os.path.dirname(here)!r}, {here!r}]; import test_gpu_step_paths as t; "
+                f"t._gradients_of_short_rows({path!r})")
+        subprocess.run([sys.executable, "-c", code], check=True, timeout=300,
+                       env=dict(os.environ, CUDA_LAUNCH_BLOCKING=wait))
+        got.append(np.load(path))
+    assert np.isfinite(got[0]).all() and np.array_equal(got[0], got[1])
