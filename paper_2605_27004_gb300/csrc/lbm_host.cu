@@ -183,6 +183,7 @@ struct lbm_ctx {
     // there by the forward run (step_held)
     long long held_t0 = -1;
     int held = 0;
+    bool captured = false;  // an lbm_step was captured by the caller: its replays advance the state unseen
     double grad_theta[6] = {0};
     double grad_tau = 0.0;
 
@@ -541,6 +542,15 @@ int record_ckpt(lbm_ctx* c) {
     LBM_CUDA(c, cudaMemcpyAsync(p, state_ptr(c), c->state_bytes(), cudaMemcpyDefault, c->stream));
     c->rec_valid = k + 1;
     return LBM_OK;
+}
+
+bool is_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
 }
 
 int check_flag(lbm_ctx* c) {
@@ -982,10 +992,13 @@ int lbm_step(lbm_ctx* c, int n) {
     long long next_check = c->opt.check_every > 0 ? (c->steps / c->opt.check_every + 1) * c->opt.check_every : -1;
     const bool recording = c->rec_K > 0 && c->rec_valid * c->rec_K > c->steps;
     long long next_rec = recording ? (c->steps / c->rec_K + 1) * c->rec_K : -1;
-    // the last segment's states stay in the adjoint's buffers where an earlier adjoint allocated them
+    // The last segment's states stay in the adjoint's buffers where an earlier adjoint allocated them. Not
+    // under a caller's capture, whose graph would keep the addresses of buffers that lbm_adjoint_release
+    // frees, nor from then on: a replay starts another trajectory without a call that drops them.
     long long hold_from = -1;
     if (n > 0) c->held = 0;
-    if (recording && n > 0 && next_check < 0 && !c->slab && c->init_fields) {
+    if (recording && n > 0 && !c->captured) c->captured = is_capturing(c->stream);
+    if (recording && n > 0 && next_check < 0 && !c->slab && c->init_fields && !c->captured) {
         const long long end = c->steps + n, t0 = (end - 1) / c->rec_K * c->rec_K;
         if (t0 >= c->steps && end - t0 >= 2 && (long long)c->adj_bufs.size() >= end - t0) {
             hold_from = t0;

@@ -228,3 +228,61 @@ def test_gradient_records_match_waited_launches(tmp_path):
                        env=dict(os.environ, CUDA_LAUNCH_BLOCKING=wait))
         got.append(np.load(path))
     assert np.isfinite(got[0]).all() and np.array_equal(got[0], got[1])
+
+
+# A caller's graph of a recorded run: it keeps no address of the adjoint's buffers, which may be released
+# before a replay, and a replay starts another trajectory without a call that says so, so that states held
+# by an earlier run must not serve its gradient.
+@pytest.mark.parametrize("storage,scheme", [("fp32s", "pull"), ("fp16s", "aa")])
+def test_recorded_run_in_a_callers_graph(storage, scheme):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    dims, n, K = (18, 7, 6), 20, 5
+    N = int(np.prod(dims))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    fields = [0.03 * torch.randn(3, N, device="cuda", generator=g) for _ in range(2)]
+    w = torch.randn(3, N, device="cuda", generator=g)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+
+    def context():
+        L = lbm.LBM(19, *dims, 0.7, rand_theta(2, 3), storage=storage, scheme=scheme, stream=s)
+        L.record_checkpoints(K)
+        return L
+
+    def gradient(L):
+        before = L.launches
+        L.adjoint(w, n, K)
+        return L.gradients(), L.launches - before
+
+    with torch.cuda.stream(s):
+        want = []
+        for u in fields:
+            L = context()
+            L.init(None, u)
+            L.step(n)
+            want.append((gradient(L), L.populations()))
+        L, u = context(), fields[0].clone()
+        for _ in range(2):  # the second run holds its last segment
+            L.init(None, u)
+            L.step(n)
+            (_, _, du0), launches = gradient(L)
+            assert torch.equal(du0, want[0][0][0][2])
+        assert launches == want[0][0][1] - (K - 1)
+        graph = torch.cuda.CUDAGraph()
+        s.synchronize()
+        with torch.cuda.graph(graph, stream=s):
+            L.init(None, u)
+            L.step(n)
+        for other in (False, True):  # without and with a run of the library's own before the replay
+            if other:
+                L.init(None, fields[0])
+                L.step(n)
+            u.copy_(fields[1])
+            graph.replay()
+            ((dth, dtau, du0), _), ref = gradient(L), want[1][0][0]
+            assert torch.equal(du0, ref[2]) and np.array_equal(dth, ref[0]) and dtau == ref[1]
+        L.adjoint_release()
+        u.copy_(fields[0])
+        graph.replay()
+        assert torch.equal(L.populations(), want[0][1])
