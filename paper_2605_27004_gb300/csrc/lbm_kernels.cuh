@@ -384,39 +384,46 @@ __device__ __forceinline__ Macro<T> bgk(const Coef<T>& cf, T (&d)[Q]) {
 
 // ---------------------------------------------------------------------------------------------
 // BGK collision of FP64 storage, in place on the stored populations f_i. The FP64 kernels are bound
-// by the FP64 pipe (two fused multiply-adds per SM and clock: 85 % busy at 64^3 with the shifted
-// form above, 263 FP64 instructions per D3Q19 cell, while DRAM is 4 % busy), so this form counts
-// operations: no shift on load and store (FP64 keeps f ~ w_i to 1e-16; om rho A_i is om feq's
-// density part and r_i at once), 1/tau folded into per-cell factors, and (c.u)^2 of axes and edges
-// from shared products (edge: u_a^2 + u_b^2 +- 2 u_a u_b; minus |u|^2 it is +- 2 u_a u_b - u_c^2).
-// About 200 a cell: D3Q19 64^3 137 -> 98.6 us a step.
+// by the FP64 pipe (two fused multiply-adds per SM and clock: 85 % busy at 64^3 with the form above,
+// 263 FP64 instructions per D3Q19 cell, while DRAM is 4 % busy), so this form counts operations: a
+// direction pair as its sum and difference, of which only the sum needs the shift by r (the difference
+// is exact); 1/tau folded into per-cell factors; and (c.u)^2 of axes and edges from shared products
+// (edge: u_a^2 + u_b^2 +- 2 u_a u_b; minus |u|^2 it is +- 2 u_a u_b - u_c^2).
+// What is relaxed are deviations from r, as everywhere: the rounding of the density part scales with
+// rho - rho0. Without the shift (some 30 operations less) it acts on the whole density and comes back
+// with the same sign every step near a steady state: in 10,000 steps that moved the mass of a box by
+// 1e-13 to 1e-12 (here below 1e-15), and after 50 steps of 16^3 velocities were 6 times further from
+// their exact values. Measured: D3Q19 64^3 137 -> 116 us a step (98 without the shift).
 // ---------------------------------------------------------------------------------------------
 template <int Q>
-__device__ __forceinline__ Macro<double> bgk_raw(const Coef<double>& cf, double (&f)[Q]) {
+__device__ __forceinline__ Macro<double> bgk64(const Coef<double>& cf, double (&f)[Q]) {
     constexpr bool D3 = Lat<Q>::D == 3;
-    double s = f[0], j[3] = {0.0, 0.0, 0.0};
+    double p[Lat<Q>::P], o[Lat<Q>::P];  // sums (of deviations) and differences of the pairs
+    const double d0 = f[0] - cf.so[0];
+    double s = d0, j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int k = 0; k < Lat<Q>::P; ++k) {
         const Vec3 v = vel<Q>(2 * k + 1);
-        const double a = f[2 * k + 1], b = f[2 * k + 2], o = a - b;
         const int n = v.x * v.x + v.y * v.y + v.z * v.z;
-        s += a + b;
+        o[k] = f[2 * k + 1] - f[2 * k + 2];
+        p[k] = fma(2.0, f[2 * k + 2] - cf.so[2 * k + 1], o[k]);  // r is the same for both
+        s += p[k];
         // the axis pairs come first and start the sums
-        if (v.x) j[0] = n == 1 ? o : (v.x > 0 ? j[0] + o : j[0] - o);
-        if (v.y) j[1] = n == 1 ? o : (v.y > 0 ? j[1] + o : j[1] - o);
-        if (v.z) j[2] = n == 1 ? o : (v.z > 0 ? j[2] + o : j[2] - o);
+        if (v.x) j[0] = n == 1 ? o[k] : (v.x > 0 ? j[0] + o[k] : j[0] - o[k]);
+        if (v.y) j[1] = n == 1 ? o[k] : (v.y > 0 ? j[1] + o[k] : j[1] - o[k]);
+        if (v.z) j[2] = n == 1 ? o[k] : (v.z > 0 ? j[2] + o[k] : j[2] - o[k]);
     }
     Macro<double> m;
-    m.rho = s;
-    m.drho = 0.0;  // not used in this form
+    m.drho = s;
+    m.rho = cf.rho0 + s;
     m.jx = j[0];
     m.jy = j[1];
     m.jz = j[2];
-    const double inv = 1.0 / s;
+    const double inv = 1.0 / m.rho;
     m.ux = j[0] * inv;
     m.uy = j[1] * inv;
     m.uz = D3 ? j[2] * inv : 0.0;
-    const double om1 = 1.0 - cf.omega, omrho = cf.omega * s;
+    const double om1 = 1.0 - cf.omega, half = 0.5 * om1, omrho = cf.omega * m.rho, omdrho = cf.omega * s;
     const double u[3] = {m.ux, m.uy, m.uz};
     const double q[3] = {u[0] * u[0], u[1] * u[1], D3 ? u[2] * u[2] : 0.0};
     const double sum[3] = {D3 ? q[1] + q[2] : q[1], D3 ? q[0] + q[2] : q[0], q[0] + q[1]};  // |u|^2 - u_a^2
@@ -427,7 +434,7 @@ __device__ __forceinline__ Macro<double> bgk_raw(const Coef<double>& cf, double 
     const double kx = fma(cf.K[0], u[0], D3 ? fma(cf.K[3], u[1], cf.K[4] * u[2]) : cf.K[3] * u[1]);
     const double ky = fma(cf.K[3], u[0], D3 ? fma(cf.K[1], u[1], cf.K[5] * u[2]) : cf.K[1] * u[1]);
     const double r45 = 4.5 * omrho, r15 = r45 * usq * (1.0 / 3.0), rc3 = cf.c3 * omrho;
-    f[0] = fma(om1, f[0], fma(omrho, cf.A[0], -(weight<Q>(0) * r15)));
+    f[0] = fma(om1, d0, fma(omdrho, cf.A[0], -(weight<Q>(0) * r15))) + cf.so[0];
 #pragma unroll
     for (int k = 0; k < Lat<Q>::P; ++k) {
         const int i = 2 * k + 1;
@@ -460,20 +467,22 @@ __device__ __forceinline__ Macro<double> bgk_raw(const Coef<double>& cf, double 
             g = uc2 - usq;
             bk = v.z > 0 ? bxy + bz : bxy - bz;
         }
-        const double E = fma(a, uc2, fma(omrho, cf.A[i], -base));
-        const double O = fma(uc, fma(b, g, omrho * cf.B[i]), -bk);
-        f[i] = fma(om1, f[i], E + O);
-        f[i + 1] = fma(om1, f[i + 1], E - O);
+        // half the relaxed sum and difference
+        const double E = fma(half, p[k], fma(a, uc2, fma(omdrho, cf.A[i], -base)));
+        const double O = fma(half, o[k], fma(uc, fma(b, g, omrho * cf.B[i]), -bk));
+        f[i] = (E + O) + cf.so[i];
+        f[i + 1] = (E - O) + cf.so[i];
     }
     return m;
 }
 
-// The collision of a flow step on gathered populations: FP64 storage as stored, the others shifted.
+// The collision of a flow step on gathered populations: FP64 storage takes them as stored, the others
+// shifted.
 template <int Q, int S>
 __device__ __forceinline__ Macro<typename Store<S>::T> collide(const Coef<typename Store<S>::T>& cf,
                                                                typename Store<S>::T (&d)[Q]) {
     if constexpr (S == 1)
-        return bgk_raw<Q>(cf, d);
+        return bgk64<Q>(cf, d);
     else
         return bgk<Q, typename Store<S>::T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
 }

@@ -1,10 +1,10 @@
 // D2Q9 FP64 steps of the smallest boxes without walls: four lanes per cell.
 //
 // A warp's FP64 instruction takes 64 clocks of its scheduler's pipe whatever its lanes hold, so a box
-// with fewer warps than the GPU has schedulers takes one warp's 95 of them, 3 us, however small it
+// with fewer warps than the GPU has schedulers takes one warp's 110 of them, 3.5 us, however small it
 // is. Here each lane owns one direction pair of a cell: the moments come from two exchanges within
-// the four lanes, and a lane evaluates the equilibrium of its pair only, about 50 instructions in
-// four times as many warps: 64^2 4.6 -> 3.85 us a step, 33 x 60 4.6 -> 3.6.
+// the four lanes, and a lane evaluates the equilibrium of its pair only, about 55 instructions in
+// four times as many warps: 64^2 5.3 -> 4.2 us a step, 33 x 60 5.3 -> 3.9.
 #pragma once
 #include "lbm_kernels.cuh"
 
@@ -16,14 +16,15 @@ __device__ __forceinline__ double sum_of_four(double v) {
     return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// bgk_raw<9> with the pair (+v, -v) of lane j in f and g (see there).
+// bgk64<9> with the pair (+v, -v) of lane j in f and g (see there).
 __device__ __forceinline__ void bgk_lane(const Coef<double>& cf, int j, double& rest, double& f, double& g, double& rho,
                                          double& usum) {
-    const double o = f - g;
-    const double s = rest + sum_of_four(f + g);
+    const double r0 = cf.so[0], r = j == 0 ? cf.so[1] : j == 1 ? cf.so[3] : j == 2 ? cf.so[5] : cf.so[7];
+    const double d0 = rest - r0, o = f - g, p = fma(2.0, g - r, o);
+    const double drho = d0 + sum_of_four(p), s = cf.rho0 + drho;
     const double jx = sum_of_four(j == 1 ? 0.0 : o), jy = sum_of_four(j == 0 ? 0.0 : j == 3 ? -o : o);
     const double inv = 1.0 / s, ux = jx * inv, uy = jy * inv;
-    const double om1 = 1.0 - cf.omega, omrho = cf.omega * s;
+    const double om1 = 1.0 - cf.omega, half = 0.5 * om1, omrho = cf.omega * s, omdrho = cf.omega * drho;
     const double usq = fma(ux, ux, uy * uy);
     const double kx = fma(cf.K[0], ux, cf.K[3] * uy), ky = fma(cf.K[3], ux, cf.K[1] * uy);
     const double r45 = 4.5 * omrho, r15 = r45 * usq * (1.0 / 3.0);
@@ -34,11 +35,11 @@ __device__ __forceinline__ void bgk_lane(const Coef<double>& cf, int j, double& 
     const double uc = (j == 1 ? 0.0 : ux) + (j == 0 ? 0.0 : j == 3 ? -uy : uy);
     const double ck = (j == 1 ? 0.0 : kx) + (j == 0 ? 0.0 : j == 3 ? -ky : ky);
     const double b = w * (cf.c3 * omrho), uc2 = uc * uc;
-    const double E = fma(w * r45, uc2, fma(omrho, A, -(w * r15)));
-    const double O = fma(uc, fma(b, uc2 - usq, omrho * B), -((b + b) * ck));
-    rest = fma(om1, rest, fma(omrho, cf.A[0], -(weight<9>(0) * r15)));
-    f = fma(om1, f, E + O);
-    g = fma(om1, g, E - O);
+    const double E = fma(half, p, fma(w * r45, uc2, fma(omdrho, A, -(w * r15))));
+    const double O = fma(half, o, fma(uc, fma(b, uc2 - usq, omrho * B), -((b + b) * ck)));
+    rest = fma(om1, d0, fma(omdrho, cf.A[0], -(weight<9>(0) * r15))) + r0;
+    f = (E + O) + r;
+    g = (E - O) + r;
     rho = s;
     usum = ux + uy;
 }

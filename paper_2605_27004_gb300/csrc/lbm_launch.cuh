@@ -103,9 +103,9 @@ struct Launch {
     // porous AA 160^3 148 -> 142, scalar 64 x 70 x 60 7.5 -> 7.1. D3Q27 boxes without walls beyond 2M cells are
     // as fast or 1 % faster with 256 outside the flow's AA steps (pull 256^3 522 against 527).
     // FP64 steps are bound by the FP64 pipes, one per scheduler of an SM, so they run single warps as
-    // blocks, which spread evenly: us a step with 32, 64, 128 and 256 threads, D2Q9 64^2 4.4, 4.4, 4.9, 8.2;
-    // 96 x 198 5.2, 5.2, 5.2, 8.6; D3Q19 33 x 29 x 41 29.7, 29.6, 36.4, 37.4; D3Q27 42 x 35 x 22 29.4, 31.2,
-    // 31.4, 41.2; from 64^3 up they are alike.
+    // blocks, which spread evenly: us a step with 32, 64, 128 and 256 threads, D2Q9 64^2 5.3, 5.2, 5.5, 9.5;
+    // 96 x 198 5.8, 5.7, 5.7, 9.5; D3Q19 33 x 29 x 41 34.3, 34.3, 42.2, 43.3; D3Q27 42 x 35 x 22 33.9, 36.0,
+    // 36.2, 47.7; from 64^3 up they are alike.
     // A box too tall for such blocks (grid.y) keeps 256.
     static Shape shape_step(const Geom& g, bool flow_aa = false) {
         const int nzp = g.nz - 2 * LBM_SLAB;
