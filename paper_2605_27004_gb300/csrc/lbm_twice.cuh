@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
 #pragma unroll
                 for (int i = 0; i < Q; ++i) d[i] = to_shifted2<S>(e[i], cf.so[i]);
                 const Macro2 m = collide_pair<Q, S>(cf, d);
-                bad |= bad1(m.rho.v.x, m.ux.v.x, m.uy.v.x, m.uz.v.x) || bad1(m.rho.v.y, m.ux.v.y, m.uy.v.y, m.uz.v.y);
+                bad |= bad_pair(m, true, true);
                 float* o = sh + r * P;
                 float* of = o + b2 * (twice_count<Q>(0) * RP);
                 float* ou = o + b3 * (twice_count<Q>(1) * RP);
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
                         d[i] = to_shifted2<S>(f2(q[0], q[second]), cf.so[i]);
                 }
                 const Macro2 m = collide_pair<Q, S>(cf, d);
-                bad |= bad1(m.rho.v.x, m.ux.v.x, m.uy.v.x, m.uz.v.x) || bad1(m.rho.v.y, m.ux.v.y, m.uy.v.y, m.uz.v.y);
+                bad |= bad_pair(m, true, wb);  // without a second cell its half mixes cells that are no neighbours
                 const uint32_t n = row_out + nxy * (uint32_t)(p - 1);
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
