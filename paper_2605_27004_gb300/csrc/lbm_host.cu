@@ -144,6 +144,7 @@ struct lbm_ctx {
 
     Geom geom{};
     Shape shape{};
+    Several several{};
     uint32_t* link = nullptr;  // per-cell link words (N), null for an all-fluid box
     long long n_fluid = 0;
     uint32_t* cell_idx = nullptr;  // with walls: fluid cells (FP16 AA) or 32-byte sectors (FP16 / FP32 pull)
@@ -416,10 +417,10 @@ cudaError_t launch_step(lbm_ctx* c, cudaStream_t s) {
 // One launch from the current state: of several steps where the context allows it and `left` (the
 // steps to the next stop) does. Returns the steps taken in *taken.
 cudaError_t launch_steps(lbm_ctx* c, cudaStream_t s, long long left, int* taken) {
-    *taken = c->kind == 0 && c->scheme == LBM_PULL2 && !c->slab ? c->ops->steps_at_once(c->geom, left) : 1;
+    *taken = c->kind == 0 && c->scheme == LBM_PULL2 && !c->slab ? c->ops->steps_at_once(c->geom, c->several, left) : 1;
     if (*taken == 1) return launch_step(c, s);
     const cudaError_t e =
-        c->ops->step_several(c->geom, c->coef(), *taken, c->pop[c->cur], c->pop[c->cur ^ 1], c->flag, s);
+        c->ops->step_several(c->geom, c->coef(), c->several, *taken, c->pop[c->cur], c->pop[c->cur ^ 1], c->flag, s);
     c->cur ^= 1;
     c->steps += *taken;
     c->launches += 1;
@@ -898,6 +899,7 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
             }
         }
     }
+    c->several = c->ops->plan_several(c->geom);
     const size_t SB = c->state_bytes();
     c->pop[0] = dev_alloc(c, SB);
     if (c->scheme == LBM_PULL2) c->pop[1] = dev_alloc(c, SB);

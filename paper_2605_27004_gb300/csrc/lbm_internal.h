@@ -96,6 +96,22 @@ inline int block_x_for(int n, int threads = 256) {
     return best;
 }
 
+// Tiles of a box in launches of two steps (lbm_twice.cuh): the x extent in `tx` tiles of `w` cells (the
+// last one may be narrower), all rows of tiles together `tiles`. Their planes are walked tile by tile:
+// block b takes the `run` planes from plane b run on of this order (chunks = 0), or one of `chunks` parts
+// of `run` planes of one tile.
+struct Tiles {
+    int w, tx, tiles, run, chunks;
+};
+
+// How a context takes several steps per launch, found once when it is made: the search for the tiles
+// tries every split of nz, 0.1 ms for the tallest boxes, more than a step takes there.
+struct Several {
+    int sms;     // SMs of the device
+    bool twice;  // two steps per launch, on `tiles`
+    Tiles tiles;
+};
+
 // Launch of a kernel that waits for the previous one itself (wait_previous) before its first access
 // to memory that another kernel writes: its blocks may be set up while that one drains.
 template <typename... P, typename... A>
@@ -159,11 +175,13 @@ struct Ops {
     // the even AA step with walls over the sector list (FP16 r-shifted storage)
     cudaError_t (*step_aa_even_sectors)(const Geom&, const void* coef, const SectorList&, const void* src, void* dst,
                                         int* flag, cudaStream_t);
-    // several flow steps of the pull scheme in one launch: `steps_at_once` says how many of `left` one
-    // launch takes (1: step_pull); src and dst are the two arrays, as for one step
-    int (*steps_at_once)(const Geom&, long long left);
-    cudaError_t (*step_several)(const Geom&, const void* coef, int steps, const void* src, void* dst, int* flag,
-                                cudaStream_t);
+    // several flow steps of the pull scheme in one launch: `plan_several` looks at the box once,
+    // `steps_at_once` says how many of `left` one launch takes (1: step_pull); src and dst are the two
+    // arrays, as for one step
+    Several (*plan_several)(const Geom&);
+    int (*steps_at_once)(const Geom&, const Several&, long long left);
+    cudaError_t (*step_several)(const Geom&, const void* coef, const Several&, int steps, const void* src, void* dst,
+                                int* flag, cudaStream_t);
 };
 
 // One translation unit per (lattice, storage): lbm_ops.cu compiled with LBM_Q / LBM_S, and for

@@ -437,19 +437,24 @@ struct Launch {
     }
     // D2Q9 FP32 storage in whole boxes (lbm_plane.cuh)
     static constexpr bool PLANE = (S == 0 || S == 2) && Q == 9;
-    static int steps_at_once(const Geom& g, long long left) {
+    static Several plan_several(const Geom& g) {
+        Several s{};
+        s.sms = sm_count();
+        if constexpr (TWICE) s.twice = !g.link && twice_pays(g, s.sms, s.tiles);
+        return s;
+    }
+    static int steps_at_once(const Geom& g, const Several& s, long long left) {
         if (g.link || left < 2) return 1;
-        if constexpr (TWICE) return twice_pays(g, sm_count()) ? 2 : 1;
-        if constexpr (PLANE) return plane_steps(g, sm_count(), left);
+        if constexpr (TWICE) return s.twice ? 2 : 1;
+        if constexpr (PLANE) return plane_steps(g, s.sms, left);
         return 1;
     }
 
-    static cudaError_t step_several(const Geom& g, const void* coef, int steps, const void* src, void* dst, int* flag,
-                                    cudaStream_t st) {
+    static cudaError_t step_several(const Geom& g, const void* coef, const Several& s, int steps, const void* src,
+                                    void* dst, int* flag, cudaStream_t st) {
         const CF& cf = *static_cast<const CF*>(coef);
         if constexpr (TWICE) {
-            long long walks = 0;
-            const Tiles t = twice_tiles(g, std::max(1, sm_count()), walks);
+            const Tiles& t = s.tiles;
             const cudaError_t e = cudaFuncSetAttribute(k_step_twice<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        twice_smem<Q>());
             if (e != cudaSuccess) return e;
@@ -459,7 +464,7 @@ struct Launch {
             return cudaGetLastError();
         }
         if constexpr (PLANE) {
-            return launch_planes<S>(g, cf, sm_count(), steps, cpl(src, g), mpl(dst, g), flag, st);
+            return launch_planes<S>(g, cf, s.sms, steps, cpl(src, g), mpl(dst, g), flag, st);
         }
         return cudaErrorNotSupported;
     }
@@ -479,7 +484,8 @@ struct Launch {
     static const Ops& ops() {
         static const Ops o = {&init,     &step_pull, &step_aa,   &step_pull_sectors, &step_aa_list, &moments,
                               &totals,   &adj_seed,  &adj_step,  &adj_init,          &link_mask,    &ade_pull,
-                              &ade_aa,   &ade_pull_sectors, &step_aa_even_sectors, &steps_at_once, &step_several};
+                              &ade_aa,   &ade_pull_sectors, &step_aa_even_sectors, &plan_several, &steps_at_once,
+                              &step_several};
         return o;
     }
 };

@@ -63,13 +63,6 @@ __host__ __device__ constexpr int twice_smem() {
            (int)sizeof(float);
 }
 
-// Tiles of the box: the x extent in `tx` tiles of `w` cells (the last one may be narrower), all rows of
-// tiles together `tiles`. Their planes are walked tile by tile: block b takes the `run` planes from
-// plane b run on of this order (chunks = 0), or one of `chunks` parts of `run` planes of one tile.
-struct Tiles {
-    int w, tx, tiles, run, chunks;
-};
-
 template <int Q, int S>
 __global__ void __launch_bounds__(TWICE_THREADS, 1)
     k_step_twice(Geom g, Coef<float> cf, Tiles t, const Planes<const float> src, const Planes<float> dst,
@@ -233,10 +226,10 @@ inline Tiles twice_tiles(const Geom& g, int slots, long long& walks) {
 // 160^3 1.00 (0.77), 144^3 0.94 (0.68). Rows that are not whole sectors make the tiles' edges share
 // sectors (257^3 0.96, 300^3 0.89), and boxes whose two states stay in L2 in good part are faster in
 // single steps (96^3 0.78).
-inline bool twice_pays(const Geom& g, int slots) {
+inline bool twice_pays(const Geom& g, int slots, Tiles& t) {
     if (g.nx % 8 != 0 || g.N < 1900000u || slots < 1) return false;
     long long walks = 0;
-    twice_tiles(g, slots, walks);
+    t = twice_tiles(g, slots, walks);
     const double full = (double)g.N / ((double)walks * slots * TWICE_W * (TWICE_ROWS - 2));
     return full >= 0.82;
 }

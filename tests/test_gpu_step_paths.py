@@ -114,6 +114,27 @@ def test_two_steps_per_launch_accept_an_uneven_state():
     assert L.moments()[0].min() > 0
 
 
+# The split of a box for two steps per launch tries every split of nz: once per context, not per launch,
+# where it cost the host 140 us at nz = 32768 (a launch costs it some 5). Enqueueing single launches takes
+# no longer in a tall box than in a flat one of as many cells.
+def test_tall_boxes_cost_the_host_no_more():
+    import time
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    took = {}
+    for dims in ((8, 32768, 8), (8, 8, 32768)):
+        L = lbm.LBM(19, *dims, 0.8, np.eye(3) / 3, use_graphs=-1)
+        L.init()
+        best = 1e9
+        for _ in range(10):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            L.step(20)
+            best = min(best, time.perf_counter() - t)
+        took[dims[2]] = best
+    assert took[32768] < 3 * took[8]
+
+
 # FP16 storage in rows of odd length, and AA with walls: two cells per thread. The FP16 form shifted by
 # the weights runs one cell per thread, and at Theta = cs2 I its stored values and its arithmetic
 # are the same, so the two give the same bits; so do pull and AA, which round the same post-collision
