@@ -184,6 +184,7 @@ struct lbm_ctx {
     // there by the forward run (step_held)
     long long held_t0 = -1;
     int held = 0;
+    long long hold_n = -1;  // the steps of the last adjoint, until a run of as many has held its states
     bool captured = false;  // an lbm_step was captured by the caller: its replays advance the state unseen
     double grad_theta[6] = {0};
     double grad_tau = 0.0;
@@ -432,7 +433,10 @@ cudaError_t launch_steps(lbm_ctx* c, cudaStream_t s, long long left, int* taken)
 // extra traffic: a step reads one array and writes another), and the last one into the context's.
 // The adjoint then starts without recomputing that segment. The buffers are those an earlier
 // lbm_adjoint allocated. Training steps, K = 20: 128^3 FP32 n = 100
-// 18.1 -> 17.3 ms, 192^3 FP16 AA n = 40 18.9 -> 16.8 ms.
+// 18.1 -> 17.3 ms, 192^3 FP16 AA n = 40 18.9 -> 16.8 ms. A run without an adjoint pays for it: its segment
+// goes through buffers of its own in single steps (256^3 368 instead of 308 us a step, D2Q9 96 x 80 1.8
+// instead of 0.8). So only a run that reaches the last adjoint's n is held, and one for each adjoint:
+// of the runs of a line search between two gradients, the first.
 int step_held(lbm_ctx* c, int len) {
     const long long t0 = c->steps;
     const void* src = state_ptr(c);
@@ -451,6 +455,7 @@ int step_held(lbm_ctx* c, int len) {
     c->steps = t0 + len;
     c->held_t0 = t0;
     c->held = len - 1;
+    c->hold_n = -1;
     return LBM_OK;
 }
 
@@ -1002,7 +1007,7 @@ int lbm_step(lbm_ctx* c, int n) {
     if (recording && n > 0 && !c->captured) c->captured = is_capturing(c->stream);
     if (recording && n > 0 && next_check < 0 && !c->slab && c->init_fields && !c->captured) {
         const long long end = c->steps + n, t0 = (end - 1) / c->rec_K * c->rec_K;
-        if (t0 >= c->steps && end - t0 >= 2 && (long long)c->adj_bufs.size() >= end - t0) {
+        if (end == c->hold_n && t0 >= c->steps && end - t0 >= 2 && (long long)c->adj_bufs.size() >= end - t0) {
             hold_from = t0;
             graphs = graphs && t0 - c->steps >= gsteps;
         }
@@ -1467,6 +1472,7 @@ int lbm_adjoint(lbm_ctx* c, const void* loss_grad, int n, int K) {
     }
     c->grad_tau = c->hout[6];
     c->grads_ready = true;
+    c->hold_n = n;
     c->last_adj_K2 = longest;
     c->last_adj_prefetch = prefetched;
     release();

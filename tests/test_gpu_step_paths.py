@@ -261,6 +261,43 @@ def test_gradient_with_held_segment(n, K, storage, scheme, graphs):
     assert again[4] == first[4] - held
 
 
+# A run whose states no gradient will read is not taken through the adjoint's buffers in single steps: not
+# the pieces of a run (D2Q9 FP32 takes 20 steps in 3 launches), not a run of other length than
+# the last gradient's, and of those that follow one gradient only the first. Launches per run, and the
+# gradient afterwards.
+def test_only_runs_before_a_gradient_are_held():
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    dims, n, K = (30, 20, 1), 40, 20
+    N = int(np.prod(dims))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    u = 0.03 * torch.randn(2, N, device="cuda", generator=g)
+    w = torch.randn(2, N, device="cuda", generator=g)
+    L = lbm.LBM(9, *dims, 0.7, rand_theta(2, 2), use_graphs=-1)
+    L.record_checkpoints(K)
+
+    def run(pieces):
+        L.init(None, u)
+        before = L.launches
+        for m in pieces:
+            L.step(m)
+        return L.launches - before
+
+    several = run([20])  # 8 + 8 + 4 steps
+    assert several == 3 and run([n]) == 2 * several
+    L.adjoint(w, n, K)
+    first = L.gradients()
+    assert run([20, 10, 5, 5]) == several + 3 + 2 + 2  # 8 + 2 * 1, 4 + 1, 4 + 1
+    assert run([25]) == several + 2
+    assert run([n]) == several + K  # held
+    assert run([n]) == 2 * several  # its states were not used
+    L.adjoint(w, n, K)
+    assert run([n]) == several + K
+    L.adjoint(w, n, K)
+    again = L.gradients()
+    assert torch.equal(again[2], first[2]) and np.array_equal(again[0], first[0]) and again[1] == first[1]
+
+
 # The adjoint's steps add to the gradient records of the step before, and are set up while that one
 # runs: their sums against those of a process that waits for every launch, bit for bit. Rows that leave
 # fewer than the eight threads of a record in the last block of a row (5, 260 and 33 cells).
