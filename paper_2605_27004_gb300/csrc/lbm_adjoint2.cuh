@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128, 5)
 #pragma unroll
         for (int k = 0; k < Lat<Q>::P; ++k) {
             drho += dk[2 * k + 1] + dk[2 * k + 2];
-            add_c2(vel<Q>(2 * k + 1), dk[2 * k + 1] - dk[2 * k + 2], jx, jy, jz);
+            add_c(vel<Q>(2 * k + 1), dk[2 * k + 1] - dk[2 * k + 2], jx, jy, jz);
         }
         const F2 rho = f2(cf.rho0) + drho;
         const F2 inv = f2(1.f / rho.v.x, 1.f / rho.v.y);
@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(128, 5)
             const Vec3 v = vel<Q>(i);
             const int cc[3] = {v.x, v.y, v.z};
             const F2 w = f2((float)weight<Q>(i));
-            const F2 uc = vdot2(v, u[0], u[1], u[2]);
-            const F2 qk = vdot2(v, kx, ky, kz);
+            const F2 uc = cdot(v, u[0], u[1], u[2]);
+            const F2 qk = cdot(v, kx, ky, kz);
             const F2 E = fma2(drho, f2(cf.A[i]), (w * r45) * fma2(uc, uc, -usq3));
             const F2 cub = fma2(uc, fma2(uc, uc, -usq), -(f2(2.f) * qk));
             const F2 O = rho * fma2(uc, f2(cf.B[i]), f2(cf.c3 * (float)weight<Q>(i)) * cub);
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(128, 5)
 #pragma unroll
         for (int k = 0; k < Lat<Q>::P; ++k) {
             const int i = 2 * k + 1;
-            const F2 cv = vdot2(vel<Q>(i), vv[0], vv[1], vv[2]);
+            const F2 cv = cdot(vel<Q>(i), vv[0], vv[1], vv[2]);
             st2(lam.p[i] + c.n, fma2(om1, mu[i], om * (v0 + cv)));
             st2(lam.p[i + 1] + c.n, fma2(om1, mu[i + 1], om * (v0 - cv)));
         }

@@ -16,74 +16,6 @@
 namespace lbm {
 inline namespace LBM_VARIANT {
 
-// bgk<Q, float, fix_momentum, fold_omega> of storage S on two cells, in the order of operations (fused
-// multiply-adds included) that the one-cell kernels are compiled to, so that both give the same bits;
-// tests/test_gpu_step_paths.py holds them to it.
-template <int Q, int S>
-__device__ __forceinline__ Macro2 collide_pair(const Coef<float>& cf, F2 (&d)[Q]) {
-    constexpr bool FOLD = Store<S>::fold_omega;
-    Macro2 m;
-    F2 s = d[0], jx = f2(0.f), jy = f2(0.f), jz = f2(0.f);
-#pragma unroll
-    for (int k = 0; k < Lat<Q>::P; ++k) {
-        const F2 a = d[2 * k + 1], b = d[2 * k + 2];
-        s += a + b;
-        add_c2(vel<Q>(2 * k + 1), a - b, jx, jy, jz);
-    }
-    m.drho = s;
-    m.rho = f2(cf.rho0) + s;
-    m.jx = jx;
-    m.jy = jy;
-    m.jz = jz;
-    const F2 inv = f2(1.f / m.rho.v.x, 1.f / m.rho.v.y);
-    m.ux = jx * inv;
-    m.uy = jy * inv;
-    m.uz = Lat<Q>::D == 3 ? jz * inv : f2(0.f);
-    const F2 usq = fma2(m.uz, m.uz, fma2(m.ux, m.ux, m.uy * m.uy));
-    const F2 nusq = -usq, nusq3 = -(usq * f2(1.0f / 3.0f));
-    // -2 K~.u
-    const F2 kx = f2(-2.f) * fma2(f2(cf.K[4]), m.uz, fma2(f2(cf.K[0]), m.ux, f2(cf.K[3]) * m.uy));
-    const F2 ky = f2(-2.f) * fma2(f2(cf.K[5]), m.uz, fma2(f2(cf.K[3]), m.ux, f2(cf.K[1]) * m.uy));
-    const F2 kz = f2(-2.f) * fma2(f2(cf.K[2]), m.uz, fma2(f2(cf.K[5]), m.uy, f2(cf.K[4]) * m.ux));
-    const F2 om = f2(cf.omega), om1 = f2(1.f - cf.omega);
-    // with FOLD 1/tau is part of the per-cell factors
-    const F2 r45 = FOLD ? om * (f2(4.5f) * m.rho) : f2(4.5f) * m.rho;
-    const F2 rho = FOLD ? om * m.rho : m.rho, drho = FOLD ? om * s : s;
-    const F2 nrho = -rho;
-    if (FOLD) {
-        d[0] = fma2(om1, d[0], fma2(drho, f2(cf.A[0]), f2((float)weight<Q>(0)) * r45 * nusq3));
-    } else {
-        const F2 rest = fma2(drho, f2(cf.A[0]), f2((float)weight<Q>(0)) * r45 * usq * f2(-1.0f / 3.0f));
-        d[0] = fma2(om1, d[0], om * rest);
-    }
-    F2 ex = -jx, ey = -jy, ez = -jz;  // post-collision momentum defect
-#pragma unroll
-    for (int k = 0; k < Lat<Q>::P; ++k) {
-        const int i = 2 * k + 1;
-        const Vec3 v = vel<Q>(i);
-        const float w = (float)weight<Q>(i);
-        const F2 uc = vdot2(v, m.ux, m.uy, m.uz);
-        const F2 nqk2 = vdot2(v, kx, ky, kz);
-        const F2 E = fma2(drho, f2(cf.A[i]), (f2(w) * r45) * fma2(uc, uc, nusq3));
-        const F2 H = fma2(uc, fma2(uc, uc, nusq), nqk2);
-        const F2 J = fma2(uc, f2(cf.B[i]), f2(w * cf.c3) * H);
-        const F2 plus = fma2(rho, J, E), minus = fma2(nrho, J, E);
-        d[i] = fma2(om1, d[i], FOLD ? plus : om * plus);
-        d[i + 1] = fma2(om1, d[i + 1], FOLD ? minus : om * minus);
-        if (Store<S>::fix_momentum) add_c2(v, d[i] - d[i + 1], ex, ey, ez);
-    }
-    if (Store<S>::fix_momentum) {
-#pragma unroll
-        for (int k = 0; k < Lat<Q>::P; ++k) {
-            const Vec3 v = vel<Q>(2 * k + 1);
-            const float c = (float)(3.0 * weight<Q>(2 * k + 1));
-            const F2 e = vdot2(v, ex, ey, ez);
-            d[2 * k + 1] = fma2(f2(-c), e, d[2 * k + 1]);
-            d[2 * k + 2] = fma2(f2(c), e, d[2 * k + 2]);
-        }
-    }
-    return m;
-}
 __device__ __forceinline__ bool bad_pair(const Macro2& m, bool a, bool b) {
     return (a && bad1(m.rho.v.x, m.ux.v.x, m.uy.v.x, m.uz.v.x)) ||
            (b && bad1(m.rho.v.y, m.ux.v.y, m.uy.v.y, m.uz.v.y));
@@ -168,7 +100,7 @@ __global__ void __launch_bounds__(CELLS2_THREADS, cells2_blocks<Q>())
     wait_previous<EARLY>();
     F2 d[Q];
     gather_cells2<Q, LAYOUT_PULL>(a, b, src, d);
-    const Macro2 m = collide_pair<Q, 3>(cf, d);
+    const Macro2 m = bgk<Q, 3>(cf, d);
     if (bad_pair(m, true, true)) *flag = 1;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -192,7 +124,7 @@ __global__ void __launch_bounds__(CELLS2_THREADS, cells2_blocks<Q>())
     wait_previous<EARLY>();
     F2 d[Q];
     gather_cells2<Q, ODD ? LAYOUT_AAODD : LAYOUT_LOCAL>(a, b, src, d);
-    const Macro2 m = collide_pair<Q, 3>(cf, d);
+    const Macro2 m = bgk<Q, 3>(cf, d);
     if (bad_pair(m, true, true)) *flag = 1;
     if (ODD) {
         forget(a);
@@ -227,7 +159,7 @@ __global__ void __launch_bounds__(CELLS2_THREADS, Q == 27 ? 5 : 6)
     F2 d[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) d[i] = ld2_rw(src.p[i] + n);
-    const Macro2 m = collide_pair<Q, 3>(cf, d);
+    const Macro2 m = bgk<Q, 3>(cf, d);
     if (bad_pair(m, fa, fb)) *flag = 1;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {

@@ -324,32 +324,9 @@ __device__ __forceinline__ T rest_eq(const Coef<T>& cf, const EqCell<T>& e) {
 }
 
 // d_i <- (1 - 1/tau) d_i + (feq_i - r_i)/tau for the equilibrium state e (Eq. LBE_BGK).
-// FOLD evaluates the same expression with 1/tau folded into the per-cell factors (om drho,
-// om rho, om 4.5 rho) and 2 K~.u precomputed, which shortens the dependency chain of every
-// population; it is used where the kernel is instruction-bound (FP16 storage; measured D3Q27
-// FP16 0.66 -> 0.70 of the copy peak) and rounds differently in the last bits.
-template <int Q, typename T, bool FOLD = false>
+template <int Q, typename T>
 __device__ __forceinline__ void relax(const Coef<T>& cf, const EqCell<T>& e, T (&d)[Q]) {
     const T om = cf.omega, om1 = T(1) - cf.omega;
-    if (FOLD) {
-        const T omdrho = om * e.drho, omrho = om * e.rho, omr45 = om * e.r45;
-        const T kx2 = T(2) * e.kx, ky2 = T(2) * e.ky, kz2 = T(2) * e.kz;
-        const T usq3 = e.usq * T(1.0 / 3.0);
-        d[0] = om1 * d[0] + (omdrho * cf.A[0] - T(weight<Q>(0)) * omr45 * usq3);
-#pragma unroll
-        for (int k = 0; k < Lat<Q>::P; ++k) {
-            const int i = 2 * k + 1;
-            const Vec3 v = vel<Q>(i);
-            const T w = T(weight<Q>(i));
-            const T uc = vdot<T>(v, e.ux, e.uy, e.uz);
-            const T qk2 = vdot<T>(v, kx2, ky2, kz2);
-            const T E = omdrho * cf.A[i] + (w * omr45) * (uc * uc - usq3);
-            const T O = omrho * (uc * cf.B[i] + (w * cf.c3) * (uc * (uc * uc - e.usq) - qk2));
-            d[i] = om1 * d[i] + (E + O);
-            d[i + 1] = om1 * d[i + 1] + (E - O);
-        }
-        return;
-    }
     d[0] = om1 * d[0] + om * rest_eq<Q, T>(cf, e);
 #pragma unroll
     for (int k = 0; k < Lat<Q>::P; ++k) {
@@ -360,23 +337,115 @@ __device__ __forceinline__ void relax(const Coef<T>& cf, const EqCell<T>& e, T (
     }
 }
 
-// BGK collision in place on shifted populations; returns the macroscopic state.
-template <int Q, typename T, bool FIX, bool FOLD = false>
-__device__ __forceinline__ Macro<T> bgk(const Coef<T>& cf, T (&d)[Q]) {
-    const Macro<T> m = macro_of<Q, T>(d, cf.rho0);
-    const EqCell<T> e = eq_cell<T>(cf, m.drho, m.rho, m.ux, m.uy, m.uz);
-    relax<Q, T, FOLD>(cf, e, d);
-    if (FIX) {
-        // post-collision momentum defect, removed along 3 w_i c_i
-        T ex = -m.jx, ey = -m.jy, ez = -m.jz;
+// A float whose operations round one by one, as the packed pairs' do (F2, lbm_pairs.cuh): the compiler
+// fuses multiplications and additions of plain floats as it likes, these only where mad() says so.
+struct F1 {
+    float v;
+};
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return {__fadd_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return {__fmul_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return {__fsub_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 operator-(F1 a) { return {-a.v}; }
+__device__ __forceinline__ F1& operator+=(F1& a, F1 b) { return a = a + b; }
+__device__ __forceinline__ F1& operator-=(F1& a, F1 b) { return a = a - b; }
+__device__ __forceinline__ F1 mad(F1 a, F1 b, F1 c) { return {__fmaf_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F1 reciprocal(F1 a) { return {__frcp_rn(a.v)}; }
+template <typename V>
+__device__ __forceinline__ V splat(float a);
+template <>
+__device__ __forceinline__ F1 splat<F1>(float a) {
+    return {a};
+}
+
+// v . (ax, ay, az), the first term taken as it is
+template <typename V>
+__device__ __forceinline__ V cdot(Vec3 v, V ax, V ay, V az) {
+    V r{};
+    bool first = true;
+    auto acc = [&](int s, V a) {
+        if (s == 0) return;
+        if (first) {
+            r = s > 0 ? a : -a;
+            first = false;
+        } else if (s > 0) {
+            r += a;
+        } else {
+            r -= a;
+        }
+    };
+    acc(v.x, ax);
+    acc(v.y, ay);
+    acc(v.z, az);
+    return r;
+}
+
+// BGK collision of FP32 arithmetic, in place on the shifted populations of one cell (V = F1) or two (F2);
+// returns the macroscopic state. Every operation is written out with its rounding, so that kernels of
+// one and of two cells per thread, and of one and of several steps per launch, give the same bits
+// whatever the compiler: tests/test_gpu_step_paths.py holds them to it.
+// FP16 storage folds 1/tau into the per-cell factors (om drho, om rho, om 4.5 rho), which shortens the
+// dependency chain of every population: its kernels are bound by issued instructions (D3Q27 0.66 ->
+// 0.70 of the copy peak).
+template <int Q, int S, typename V>
+__device__ __forceinline__ Macro<V> bgk(const Coef<float>& cf, V (&d)[Q]) {
+    constexpr bool FOLD = Store<S>::fold_omega;
+    Macro<V> m;
+    V s = d[0], jx = splat<V>(0.f), jy = splat<V>(0.f), jz = splat<V>(0.f);
 #pragma unroll
-        for (int k = 0; k < Lat<Q>::P; ++k) add_c<T>(vel<Q>(2 * k + 1), d[2 * k + 1] - d[2 * k + 2], ex, ey, ez);
+    for (int k = 0; k < Lat<Q>::P; ++k) {
+        const V a = d[2 * k + 1], b = d[2 * k + 2];
+        s += a + b;
+        add_c(vel<Q>(2 * k + 1), a - b, jx, jy, jz);
+    }
+    m.drho = s;
+    m.rho = splat<V>(cf.rho0) + s;
+    m.jx = jx;
+    m.jy = jy;
+    m.jz = jz;
+    const V inv = reciprocal(m.rho);
+    m.ux = jx * inv;
+    m.uy = jy * inv;
+    m.uz = Lat<Q>::D == 3 ? jz * inv : splat<V>(0.f);
+    const V usq = mad(m.uz, m.uz, mad(m.ux, m.ux, m.uy * m.uy));
+    const V nusq = -usq, nusq3 = -(usq * splat<V>(1.0f / 3.0f));
+    // -2 K~.u
+    const V kx = splat<V>(-2.f) * mad(splat<V>(cf.K[4]), m.uz, mad(splat<V>(cf.K[0]), m.ux, splat<V>(cf.K[3]) * m.uy));
+    const V ky = splat<V>(-2.f) * mad(splat<V>(cf.K[5]), m.uz, mad(splat<V>(cf.K[3]), m.ux, splat<V>(cf.K[1]) * m.uy));
+    const V kz = splat<V>(-2.f) * mad(splat<V>(cf.K[2]), m.uz, mad(splat<V>(cf.K[5]), m.uy, splat<V>(cf.K[4]) * m.ux));
+    const V om = splat<V>(cf.omega), om1 = splat<V>(1.f - cf.omega);
+    const V r45 = FOLD ? om * (splat<V>(4.5f) * m.rho) : splat<V>(4.5f) * m.rho;
+    const V rho = FOLD ? om * m.rho : m.rho, drho = FOLD ? om * s : s;
+    const V nrho = -rho;
+    if (FOLD) {
+        d[0] = mad(om1, d[0], mad(drho, splat<V>(cf.A[0]), splat<V>((float)weight<Q>(0)) * r45 * nusq3));
+    } else {
+        const V rest = mad(drho, splat<V>(cf.A[0]), splat<V>((float)weight<Q>(0)) * r45 * usq * splat<V>(-1.0f / 3.0f));
+        d[0] = mad(om1, d[0], om * rest);
+    }
+    V ex = -jx, ey = -jy, ez = -jz;  // post-collision momentum defect
+#pragma unroll
+    for (int k = 0; k < Lat<Q>::P; ++k) {
+        const int i = 2 * k + 1;
+        const Vec3 v = vel<Q>(i);
+        const float w = (float)weight<Q>(i);
+        const V uc = cdot(v, m.ux, m.uy, m.uz);
+        const V nqk2 = cdot(v, kx, ky, kz);
+        const V E = mad(drho, splat<V>(cf.A[i]), (splat<V>(w) * r45) * mad(uc, uc, nusq3));
+        const V H = mad(uc, mad(uc, uc, nusq), nqk2);
+        const V J = mad(uc, splat<V>(cf.B[i]), splat<V>(__fmul_rn(w, cf.c3)) * H);
+        const V plus = mad(rho, J, E), minus = mad(nrho, J, E);
+        d[i] = mad(om1, d[i], FOLD ? plus : om * plus);
+        d[i + 1] = mad(om1, d[i + 1], FOLD ? minus : om * minus);
+        if (Store<S>::fix_momentum) add_c(v, d[i] - d[i + 1], ex, ey, ez);
+    }
+    if (Store<S>::fix_momentum) {  // removed along 3 w_i c_i
 #pragma unroll
         for (int k = 0; k < Lat<Q>::P; ++k) {
             const Vec3 v = vel<Q>(2 * k + 1);
-            const T corr = T(3.0 * weight<Q>(2 * k + 1)) * vdot<T>(v, ex, ey, ez);
-            d[2 * k + 1] -= corr;
-            d[2 * k + 2] += corr;
+            const float c = (float)(3.0 * weight<Q>(2 * k + 1));
+            const V e = cdot(v, ex, ey, ez);
+            d[2 * k + 1] = mad(splat<V>(-c), e, d[2 * k + 1]);
+            d[2 * k + 2] = mad(splat<V>(c), e, d[2 * k + 2]);
         }
     }
     return m;
@@ -481,10 +550,17 @@ __device__ __forceinline__ Macro<double> bgk64(const Coef<double>& cf, double (&
 template <int Q, int S>
 __device__ __forceinline__ Macro<typename Store<S>::T> collide(const Coef<typename Store<S>::T>& cf,
                                                                typename Store<S>::T (&d)[Q]) {
-    if constexpr (S == 1)
+    if constexpr (S == 1) {
         return bgk64<Q>(cf, d);
-    else
-        return bgk<Q, typename Store<S>::T, Store<S>::fix_momentum, Store<S>::fold_omega>(cf, d);
+    } else {
+        F1 e[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) e[i].v = d[i];
+        const Macro<F1> m = bgk<Q, S>(cf, e);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) d[i] = e[i].v;
+        return {m.drho.v, m.rho.v, m.jx.v, m.jy.v, m.jz.v, m.ux.v, m.uy.v, m.uz.v};
+    }
 }
 // the stored value of a collided population
 template <int S>

@@ -40,32 +40,11 @@ __device__ __forceinline__ F2& operator-=(F2& a, F2 b) {
     return a;
 }
 
-__device__ __forceinline__ void add_c2(Vec3 v, F2 val, F2& x, F2& y, F2& z) {
-    if (v.x == 1) x += val;
-    if (v.x == -1) x -= val;
-    if (v.y == 1) y += val;
-    if (v.y == -1) y -= val;
-    if (v.z == 1) z += val;
-    if (v.z == -1) z -= val;
-}
-__device__ __forceinline__ F2 vdot2(Vec3 v, F2 ax, F2 ay, F2 az) {
-    F2 r = f2(0.f);
-    bool first = true;
-    auto acc = [&](int s, F2 a) {
-        if (s == 0) return;
-        if (first) {
-            r = s > 0 ? a : -a;
-            first = false;
-        } else if (s > 0) {
-            r += a;
-        } else {
-            r -= a;
-        }
-    };
-    acc(v.x, ax);
-    acc(v.y, ay);
-    acc(v.z, az);
-    return r;
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ F2 reciprocal(F2 a) { return f2(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
+template <>
+__device__ __forceinline__ F2 splat<F2>(float a) {
+    return f2(a);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -152,9 +131,7 @@ __device__ __forceinline__ F2 gather_pair(const typename Store<S>::type* p, uint
 // differs from the one-cell kernels in the last bits; the shorter per-pair dependency chains are
 // worth 0.745 -> 0.82 of the copy peak at 256^3 for FP16 storage (measured).
 // ---------------------------------------------------------------------------------------------
-struct Macro2 {
-    F2 drho, rho, jx, jy, jz, ux, uy, uz;
-};
+using Macro2 = Macro<F2>;
 
 // Relaxation of a pair towards feq(rho, u) in shifted variables (drho = rho - rho0), with 1/tau
 // folded into the per-cell factors and 2 K~.u precomputed (see the file comment).
@@ -178,8 +155,8 @@ __device__ __forceinline__ void relax2(const Coef<float>& cf, F2 drho, F2 rho, F
         const int i = 2 * k + 1;
         const Vec3 v = vel<Q>(i);
         const F2 w = f2((float)weight<Q>(i));
-        const F2 uc = vdot2(v, ux, uy, uz);
-        const F2 qk2 = vdot2(v, kx2, ky2, kz2);
+        const F2 uc = cdot(v, ux, uy, uz);
+        const F2 qk2 = cdot(v, kx2, ky2, kz2);
         const F2 E = fma2(omdrho, f2(cf.A[i]), (w * omr45) * fma2(uc, uc, -usq3));
         const F2 cub = fma2(uc, fma2(uc, uc, -usq), -qk2);
         const F2 O = omrho * fma2(uc, f2(cf.B[i]), f2(cf.c3 * (float)weight<Q>(i)) * cub);
@@ -196,7 +173,7 @@ __device__ __forceinline__ Macro2 bgk2(const Coef<float>& cf, F2 (&d)[Q]) {
     for (int k = 0; k < Lat<Q>::P; ++k) {
         const F2 a = d[2 * k + 1], b = d[2 * k + 2];
         s += a + b;
-        add_c2(vel<Q>(2 * k + 1), a - b, jx, jy, jz);
+        add_c(vel<Q>(2 * k + 1), a - b, jx, jy, jz);
     }
     m.drho = s;
     m.rho = f2(cf.rho0) + s;
@@ -211,11 +188,11 @@ __device__ __forceinline__ Macro2 bgk2(const Coef<float>& cf, F2 (&d)[Q]) {
     if (FIX) {
         F2 ex = -m.jx, ey = -m.jy, ez = -m.jz;
 #pragma unroll
-        for (int k = 0; k < Lat<Q>::P; ++k) add_c2(vel<Q>(2 * k + 1), d[2 * k + 1] - d[2 * k + 2], ex, ey, ez);
+        for (int k = 0; k < Lat<Q>::P; ++k) add_c(vel<Q>(2 * k + 1), d[2 * k + 1] - d[2 * k + 2], ex, ey, ez);
 #pragma unroll
         for (int k = 0; k < Lat<Q>::P; ++k) {
             const Vec3 v = vel<Q>(2 * k + 1);
-            const F2 corr = f2((float)(3.0 * weight<Q>(2 * k + 1))) * vdot2(v, ex, ey, ez);
+            const F2 corr = f2((float)(3.0 * weight<Q>(2 * k + 1))) * cdot(v, ex, ey, ez);
             d[2 * k + 1] -= corr;
             d[2 * k + 2] += corr;
         }

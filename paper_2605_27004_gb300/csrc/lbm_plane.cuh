@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(THREADS)
             const Vec3 v = vel<9>(i);
             d[i] = to_shifted2<S>(f2(src.p[i][a.from(v)], src.p[i][b.from(v)]), cf.so[i]);
         }
-        const Macro2 m = collide_pair<9, S>(cf, d);
+        const Macro2 m = bgk<9, S>(cf, d);
         bad |= bad_pair(m, true, true);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(THREADS)
                 const float* q = from + i * E - v.y * EW - v.x;
                 d[i] = to_shifted2<S>(f2(q[na], q[nb]), cf.so[i]);
             }
-            const Macro2 m = collide_pair<9, S>(cf, d);
+            const Macro2 m = bgk<9, S>(cf, d);
             bad |= bad_pair(m, true, true);
             if (t < T) {
 #pragma unroll

@@ -22,7 +22,7 @@
 // 512^3: 2952 -> 2309 us a step. D3Q27 (7 rows at 254 registers, 507 to 529 against 521 us) gains
 // nothing and stays at one step a launch.
 //
-// The arithmetic is that of the one-cell kernels operation for operation (collide_pair), so that two
+// The arithmetic is that of the one-cell kernels operation for operation (bgk), so that two
 // steps in one launch give the bits of two launches.
 #pragma once
 #include "lbm_cells2.cuh"
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
                 F2 d[Q];
 #pragma unroll
                 for (int i = 0; i < Q; ++i) d[i] = to_shifted2<S>(e[i], cf.so[i]);
-                const Macro2 m = collide_pair<Q, S>(cf, d);
+                const Macro2 m = bgk<Q, S>(cf, d);
                 bad |= bad_pair(m, true, true);
                 float* o = sh + r * P;
                 float* of = o + b2 * (twice_count<Q>(0) * RP);
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(TWICE_THREADS, 1)
                     else
                         d[i] = to_shifted2<S>(f2(q[0], q[second]), cf.so[i]);
                 }
-                const Macro2 m = collide_pair<Q, S>(cf, d);
+                const Macro2 m = bgk<Q, S>(cf, d);
                 bad |= bad_pair(m, true, wb);  // without a second cell its half mixes cells that are no neighbours
                 const uint32_t n = row_out + nxy * (uint32_t)(p - 1);
 #pragma unroll
