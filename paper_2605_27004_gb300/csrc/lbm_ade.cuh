@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256)
     if (!valid) n = L.n_begin;
     Cell c;
     make_cell_index(g, L, n, c);
-    const uint32_t lw = valid ? __ldg(L.link + t) : LINK_SOLID;
+    const uint32_t lw = valid ? listed_link<S>(g, L, t, c.n) : LINK_SOLID;
     const bool solid = (lw & LINK_SOLID) != 0u;
     const unsigned act = __activemask();
     if (__all_sync(act, solid)) return;

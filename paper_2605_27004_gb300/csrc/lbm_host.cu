@@ -149,7 +149,7 @@ struct lbm_ctx {
     long long n_fluid = 0;
     uint32_t* cell_idx = nullptr;  // with walls: fluid cells (FP16 AA) or 32-byte sectors (FP16 / FP32 pull)
     CellList cells{};
-    uint32_t* cell_link = nullptr;  // their link words
+    uint32_t* cell_link = nullptr;  // FP16: their link words
     size_t cell_link_bytes = 0;
     uint2* sectors = nullptr;  // with walls, FP16 AA: the even step's sectors
     SectorList sector_list{};
@@ -869,12 +869,14 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
                 e = cudaMemcpy(c->cell_idx, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice);
                 if (e != cudaSuccess) return bail(cuda_fail(c, e, "fluid-cell list upload"));
                 c->cells.idx = c->cell_idx;
-                const uint32_t G = c->scheme == LBM_AA ? 1 : fp16 ? 16 : 8;  // cells of an entry
-                c->cell_link_bytes = idx.size() * G * 4 + 4;
-                c->cell_link = (uint32_t*)dev_alloc(c, c->cell_link_bytes);
-                if (!c->cell_link) return bail(fail(c, LBM_ERR_OOM, "listed link words"));
-                c->cells.link = c->cell_link;
-                if (!idx.empty()) {
+                const uint32_t G = c->scheme == LBM_AA ? 1 : 16;  // FP16 cells of an entry
+                if (fp16) {
+                    c->cell_link_bytes = idx.size() * G * 4 + 4;
+                    c->cell_link = (uint32_t*)dev_alloc(c, c->cell_link_bytes);
+                    if (!c->cell_link) return bail(fail(c, LBM_ERR_OOM, "listed link words"));
+                    c->cells.link = c->cell_link;
+                }
+                if (fp16 && !idx.empty()) {
                     const unsigned long long total = idx.size() * (unsigned long long)G;
                     k_list_links<<<(unsigned)std::min<unsigned long long>((total + 255) / 256, 8 * 152), 256, 0, c->stream>>>(
                         c->cell_idx, idx.size(), G, c->geom.N, c->link, c->cell_link);

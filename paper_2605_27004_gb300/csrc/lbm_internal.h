@@ -26,12 +26,13 @@ constexpr uint32_t LINK_SOLID = 0x80000000u;
 // FP32 cells (one 32-byte sector of a plane) that hold at least one fluid cell (rows of the porous
 // medium are about 30 % solid, and a lane of a solid cell still issues every instruction of its
 // warp). A cell's coordinates come back from its index by exact reciprocal multiplication:
-// n / d = umul64hi(n, ceil(2^64 / d)) for n, d < 2^32 and d >= 2. The link words stand beside the list, so
-// that a lane fetches them together with its entry and not after it (porous D3Q27 256^3, FP16: pull
-// 450 -> 429, AA 361 -> 349 us a step).
+// n / d = umul64hi(n, ceil(2^64 / d)) for n, d < 2^32 and d >= 2. With FP16 storage the link words stand
+// beside the list, so that a lane fetches them together with its entry and not after it (porous D3Q27
+// 256^3: pull 450 -> 429, AA 361 -> 349 us a step); they take 4 bytes a listed cell more. FP32 steps wait
+// for DRAM instead (500 -> 497 us), and their boxes, which may fill the GPU's memory, keep it.
 struct CellList {
     const uint32_t* idx;
-    const uint32_t* link;  // the link words of the listed cells (all cells of a listed sector), in list order
+    const uint32_t* link;  // FP16: the link words of the listed cells (all of a listed sector), in list order
     uint32_t count;
     unsigned long long rnx, rnxy;  // ceil(2^64 / nx), ceil(2^64 / (nx ny))
     uint32_t n_begin, n_end;       // the processed cells (interior planes): n_begin <= n < n_end

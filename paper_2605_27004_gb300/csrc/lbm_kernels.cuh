@@ -734,6 +734,12 @@ __device__ __forceinline__ bool make_cell_list(const Geom& g, const CellList& L,
     return true;
 }
 
+// The link word of cell n, cell t of the list (CellList).
+template <int S>
+__device__ __forceinline__ uint32_t listed_link(const Geom& g, const CellList& L, uint32_t t, uint32_t n) {
+    return __ldg(sizeof(typename Store<S>::type) == 2 ? L.link + t : g.link + n);
+}
+
 // Pull step over the list of 32-byte sectors (16 FP16 or 8 FP32 cells of a plane) that hold a
 // fluid cell: G consecutive lanes take one sector, so a warp never spends lanes on sectors of solid
 // cells only (11 % of the FP16 sectors of the porous medium, against 2 % of whole solid warps in
@@ -755,7 +761,7 @@ __global__ void __launch_bounds__(256) k_step_pull_sectors(Geom g, Coef<typename
     if (!valid) n = L.n_begin;
     Cell c;
     make_cell_index(g, L, n, c);
-    const uint32_t lw = valid ? __ldg(L.link + t) : LINK_SOLID;
+    const uint32_t lw = valid ? listed_link<S>(g, L, t, c.n) : LINK_SOLID;
     const bool solid = (lw & LINK_SOLID) != 0u;
     const unsigned act = __activemask();
     if (__all_sync(act, solid)) return;

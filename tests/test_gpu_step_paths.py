@@ -195,6 +195,16 @@ def test_steps_of_a_plane_match_single_steps(dims, storage):
         assert torch.equal(f, runs[0][1]) and torch.equal(s, runs[0][2])
 
 
+# A D3Q27 FP32 box with walls may fill the GPU's memory: beside its two arrays, a link word a cell and a list
+# entry per eight cells it takes no more than its block records (64 bytes per 256 cells).
+def test_fp32_walls_take_one_link_word_a_cell():
+    from paper_2605_27004_gb300 import lbm
+    dims = (64, 64, 64)
+    N = int(np.prod(dims))
+    L = lbm.LBM(27, *dims, 0.7, np.eye(3) / 3, solid=inputs.random_mask(N, 0.2, 4))
+    assert L.device_bytes <= N * (2 * 27 * 4 + 4 + 4 / 8 + 64 / 256) + 4096
+
+
 def test_slab_group_waits_for_fields_of_the_callers_stream():
     """SlabGroup reads the slabs' fields on the slabs' streams: the kernels that cut them out of the box on
     the caller's stream (held back here by bounded spins of some 10 ms) have to end first."""
