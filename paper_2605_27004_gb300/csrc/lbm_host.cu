@@ -741,12 +741,14 @@ void lbm_destroy(lbm_ctx* c) {
     delete c;
 }
 
-int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau, const double* Theta,
-                  const uint8_t* solid_mask, const lbm_options* opt) {
+// A context of either kind (lbm_create_ex, lbm_ade_create).
+static int create_ctx(lbm_ctx** out, int kind, int lattice, int nx, int ny, int nz, double tau, const double* Theta,
+                      const uint8_t* solid_mask, const lbm_options* opt) {
     if (!out) return LBM_ERR_INVALID_ARG;
     *out = nullptr;
     lbm_ctx* c = new (std::nothrow) lbm_ctx();
     if (!c) return LBM_ERR_OOM;
+    c->kind = kind;
     auto bail = [&](int code) {
         std::string keep = c->err;
         lbm_destroy(c);
@@ -847,7 +849,10 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
             // the grid.
             const bool fp16 = c->storage == LBM_FP16_SHIFTED || c->storage == LBM_FP16_WSHIFTED;
             const bool fp32 = c->storage == LBM_FP32 || c->storage == LBM_FP32_SHIFTED;
-            if ((fp16 || (fp32 && c->q == 27 && c->scheme == LBM_PULL2)) && nx >= 2) {
+            // The scalar's AA steps run over the grid, too.
+            const bool listed = fp16 ? c->kind == 0 || c->scheme == LBM_PULL2
+                                     : fp32 && c->q == 27 && c->scheme == LBM_PULL2;
+            if (listed && nx >= 2) {
                 std::vector<uint32_t> idx;
                 const long long z0 = c->slab ? 1 : 0;
                 const long long nb = z0 * plane, ne = (z0 + nz) * plane;
@@ -889,7 +894,7 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
                 c->cells.rnxy = ~0ULL / (unsigned long long)plane + 1ULL;
                 c->cells.n_begin = (uint32_t)nb;
                 c->cells.n_end = (uint32_t)ne;
-                if (c->scheme == LBM_AA && c->storage == LBM_FP16_SHIFTED && c->kind == 0 && c->N % 2 == 0) {
+                if (c->scheme == LBM_AA && c->storage == LBM_FP16_SHIFTED && c->N % 2 == 0) {
                     std::vector<uint2> sec;
                     for (long long n0 = 0; n0 < c->N; n0 += 16) {
                         uint32_t bits = 0;
@@ -931,6 +936,11 @@ int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau
         return bail(cuda_fail(c, cudaGetLastError(), "buffer clear"));
     *out = c;
     return LBM_OK;
+}
+
+int lbm_create_ex(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau, const double* Theta,
+                  const uint8_t* solid_mask, const lbm_options* opt) {
+    return create_ctx(out, 0, lattice, nx, ny, nz, tau, Theta, solid_mask, opt);
 }
 
 int lbm_create(lbm_ctx** out, int lattice, int nx, int ny, int nz, double tau, const double* Theta,
@@ -1648,13 +1658,7 @@ int lbm_ade_create(lbm_ctx** out, int lattice, int nx, int ny, int nz, double ta
         if (out) *out = nullptr;
         return LBM_ERR_INVALID_ARG;
     }
-    const int rc = lbm_create_ex(out, lattice, nx, ny, nz, tau, Theta, solid_mask, opt);
-    if (rc == LBM_OK) {
-        lbm_ctx* c = *out;
-        c->kind = 1;
-        if (c->scheme != LBM_PULL2) drop_lists(c);  // the scalar's AA steps run over the grid
-    }
-    return rc;
+    return create_ctx(out, 1, lattice, nx, ny, nz, tau, Theta, solid_mask, opt);
 }
 
 static int ade_field(lbm_ctx* c) {

@@ -205,6 +205,20 @@ def test_fp32_walls_take_one_link_word_a_cell():
     assert L.device_bytes <= N * (2 * 27 * 4 + 4 + 4 / 8 + 64 / 256) + 4096
 
 
+# The scalar's AA steps run over the grid: making such a context with walls takes no list memory, not even
+# for a while (8 bytes a fluid cell). Beside what it keeps there is the byte mask, and blocks are rounded.
+def test_scalar_in_place_makes_no_lists():
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    dims = (64, 64, 64)
+    N = int(np.prod(dims))
+    solid = inputs.random_mask(N, 0.2, 4)
+    torch.cuda.reset_peak_memory_stats()
+    before = torch.cuda.memory_allocated()
+    A = lbm.ADE(19, *dims, 0.7, np.eye(3) / 3, solid=solid, storage="fp16s", scheme="aa")
+    assert torch.cuda.max_memory_allocated() - before <= A.device_bytes + N + 65536
+
+
 def test_slab_group_waits_for_fields_of_the_callers_stream():
     """SlabGroup reads the slabs' fields on the slabs' streams: the kernels that cut them out of the box on
     the caller's stream (held back here by bounded spins of some 10 ms) have to end first."""
