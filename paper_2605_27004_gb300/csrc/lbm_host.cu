@@ -202,7 +202,6 @@ struct lbm_ctx {
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     long long graph_launches = 0;  // kernels of one replay
-    bool graph_flips = false;      // a replay leaves the state in the other array
 
     // checkpoints recorded during the forward run (state at t = k * rec_K)
     int rec_K = 0;
@@ -471,7 +470,6 @@ int ensure_graph(lbm_ctx* c, int gsteps) {
     for (int k = 0, taken = 0; k < gsteps && le == cudaSuccess; k += taken)
         le = launch_steps(c, c->cap_stream, gsteps - k, &taken);
     c->graph_launches = c->launches - launches0;
-    c->graph_flips = c->cur != cur0;
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
     c->cur = cur0;
@@ -1006,7 +1004,7 @@ int lbm_record_checkpoints(lbm_ctx* c, int checkpoint_every) {
 int lbm_step(lbm_ctx* c, int n) {
     if (!c || n < 0) return LBM_ERR_INVALID_ARG;
     if (!c->state_valid) return fail(c, LBM_ERR_STATE, "lbm_step before lbm_init");
-    const int gsteps = 16;
+    const int gsteps = 16;  // in 16, 8, 4 or 2 launches: an even number, so a replay leaves cur as it was
     bool graphs = !c->slab && (c->opt.use_graphs > 0 || (c->opt.use_graphs == 0 && c->N <= (1LL << 21)));
     long long next_check = c->opt.check_every > 0 ? (c->steps / c->opt.check_every + 1) * c->opt.check_every : -1;
     const bool recording = c->rec_K > 0 && c->rec_valid * c->rec_K > c->steps;
@@ -1039,7 +1037,6 @@ int lbm_step(lbm_ctx* c, int n) {
             LBM_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
             c->steps += gsteps;
             c->launches += c->graph_launches;
-            if (c->graph_flips) c->cur ^= 1;
             left -= gsteps;
             ran = true;
         }

@@ -767,9 +767,9 @@ __global__ void __launch_bounds__(256) k_step_pull_sectors(Geom g, Coef<typename
     if (__all_sync(act, solid)) return;
     T d[Q];
     if (__all_sync(act, lw == 0u)) {
-        gather<Q, S, false, LAYOUT_PULL, true, S == 1>(c, 0u, cf, src, d);
+        gather<Q, S, false, LAYOUT_PULL, true>(c, 0u, cf, src, d);
     } else if (!solid) {
-        gather<Q, S, true, LAYOUT_PULL, true, S == 1>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_PULL, true>(c, lw, cf, src, d);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = T(0);
@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(256) k_step_pull_sectors(Geom g, Coef<typename
     const bool store = store_group<typename Store<S>::type>(act, solid);
     if (!valid || !store) return;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : stored<S>(d[i], cf.so[i]));
+    for (int i = 0; i < Q; ++i) st_raw(dst.p[i] + c.n, solid ? T(0) : from_shifted<S>(d[i], cf.so[i]));
 }
 
 template <int Q, int S, int ODD>
@@ -795,20 +795,20 @@ __global__ void __launch_bounds__(256, 4) k_step_aa_list(Geom g, Coef<typename S
     const bool clean = __all_sync(__activemask(), lw == 0u);
     if (clean) {
         if (ODD)
-            gather<Q, S, false, LAYOUT_AAODD, false, S == 1>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_AAODD, false>(c, 0u, cf, src, d);
         else
-            gather<Q, S, false, LAYOUT_LOCAL, false, S == 1>(c, 0u, cf, src, d);
+            gather<Q, S, false, LAYOUT_LOCAL, false>(c, 0u, cf, src, d);
     } else if (ODD) {
-        gather<Q, S, true, LAYOUT_AAODD, false, S == 1>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_AAODD, false>(c, lw, cf, src, d);
     } else {
-        gather<Q, S, true, LAYOUT_LOCAL, false, S == 1>(c, lw, cf, src, d);
+        gather<Q, S, true, LAYOUT_LOCAL, false>(c, lw, cf, src, d);
     }
     const Macro<T> m = collide<Q, S>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
-        aa_store<Q, S, false, ODD, S == 1>(c, 0u, cf, dst, d);
+        aa_store<Q, S, false, ODD>(c, 0u, cf, dst, d);
     else
-        aa_store<Q, S, true, ODD, S == 1>(c, lw, cf, dst, d);
+        aa_store<Q, S, true, ODD>(c, lw, cf, dst, d);
 }
 
 // ---------------------------------------------------------------------------------------------

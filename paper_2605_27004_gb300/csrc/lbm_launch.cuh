@@ -34,15 +34,17 @@ struct Launch {
     // D3Q27 beyond 60 (FP32 96 x 70 x 60 11.9 -> 12.1).
     static bool early(const Geom& g, dim3 grid) {
         const unsigned long long bytes = 2ull * Q * sizeof(ST) * g.N;
-        if (S == 1 || g.N > (1u << 21) || bytes > (Q == 27 ? 60000000ull : S == 3 ? 90000000ull : ~0ull)) return false;
+        if (g.N > (1u << 21) || bytes > (Q == 27 ? 60000000ull : S == 3 ? 90000000ull : ~0ull)) return false;
         const unsigned long long blocks = (unsigned long long)grid.x * grid.y * grid.z, sms = (unsigned)sm_count();
         return blocks <= sms || blocks >= (Q == 27 && S == 3 ? 4 : 3) * sms;
     }
 #define LBM_UNWRAP(...) __VA_ARGS__
 #define LBM_EARLY(K, PARAMS, GRID, BLOCK, ...)                                                     \
     do {                                                                                           \
-        if (early(g, GRID))                                                                        \
-            return launch_after(K<LBM_UNWRAP PARAMS, true>, GRID, BLOCK, st, __VA_ARGS__);         \
+        if constexpr (S != 1) {                                                                    \
+            if (early(g, GRID))                                                                    \
+                return launch_after(K<LBM_UNWRAP PARAMS, true>, GRID, BLOCK, st, __VA_ARGS__);     \
+        }                                                                                          \
         K<LBM_UNWRAP PARAMS, false><<<GRID, BLOCK, 0, st>>>(__VA_ARGS__);                          \
     } while (0)
 
@@ -217,27 +219,35 @@ struct Launch {
         return cudaGetLastError();
     }
 
+    // the storages and lattices whose contexts with walls have a sector list (lbm_create_ex)
+    static constexpr bool SECTORS = sizeof(ST) == 2 || (Q == 27 && sizeof(ST) == 4);
     static cudaError_t step_pull_sectors(const Geom& g, const void* coef, const CellList& L, const void* src,
                                          void* dst, int* flag, cudaStream_t st) {
-        if (L.count == 0) return cudaSuccess;
-        const CF& cf = *static_cast<const CF*>(coef);
-        const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
-        const unsigned bt = pull_list_threads(threads);
-        k_step_pull_sectors<Q, S><<<(unsigned)((threads + bt - 1) / bt), bt, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g),
-                                                                                      flag);
-        return cudaGetLastError();
+        if constexpr (SECTORS) {
+            if (L.count == 0) return cudaSuccess;
+            const CF& cf = *static_cast<const CF*>(coef);
+            const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
+            const unsigned bt = pull_list_threads(threads);
+            k_step_pull_sectors<Q, S><<<(unsigned)((threads + bt - 1) / bt), bt, 0, st>>>(g, cf, L, cpl(src, g),
+                                                                                          mpl(dst, g), flag);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
     }
 
     static cudaError_t step_aa_list(const Geom& g, const void* coef, const CellList& L, int odd, const void* src,
                                     void* dst, int* flag, cudaStream_t st) {
-        if (L.count == 0) return cudaSuccess;
-        const CF& cf = *static_cast<const CF*>(coef);
-        const unsigned nb = (L.count + LIST_THREADS - 1) / LIST_THREADS;
-        if (odd)
-            k_step_aa_list<Q, S, 1><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
-        else
-            k_step_aa_list<Q, S, 0><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
-        return cudaGetLastError();
+        if constexpr (sizeof(ST) == 2) {
+            if (L.count == 0) return cudaSuccess;
+            const CF& cf = *static_cast<const CF*>(coef);
+            const unsigned nb = (L.count + LIST_THREADS - 1) / LIST_THREADS;
+            if (odd)
+                k_step_aa_list<Q, S, 1><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
+            else
+                k_step_aa_list<Q, S, 0><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, cpl(src, g), mpl(dst, g), flag);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
     }
 
 // Expands to the three layouts times mask / no mask for a kernel template K<Q, S, MASK, LAYOUT>.
@@ -415,13 +425,16 @@ struct Launch {
 
     static cudaError_t ade_pull_sectors(const Geom& g, const void* coef, const CellList& L, const void* u,
                                         const void* src, void* dst, int* flag, cudaStream_t st) {
-        if (L.count == 0) return cudaSuccess;
-        const CF& cf = *static_cast<const CF*>(coef);
-        const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
-        k_ade_pull_sectors<Q, S><<<(unsigned)((threads + LIST_THREADS - 1) / LIST_THREADS), LIST_THREADS, 0, st>>>(g,
-                    cf, L, vel_field(u, g),
-                                                                                   cpl(src, g), mpl(dst, g), flag);
-        return cudaGetLastError();
+        if constexpr (SECTORS) {
+            if (L.count == 0) return cudaSuccess;
+            const CF& cf = *static_cast<const CF*>(coef);
+            const unsigned long long threads = (unsigned long long)L.count * (32ull / sizeof(ST));  // a sector each
+            const unsigned nb = (unsigned)((threads + LIST_THREADS - 1) / LIST_THREADS);
+            k_ade_pull_sectors<Q, S><<<nb, LIST_THREADS, 0, st>>>(g, cf, L, vel_field(u, g), cpl(src, g), mpl(dst, g),
+                                                                  flag);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
     }
 
     // FP32 storage on D3Q19 in whole boxes (lbm_twice.cuh)
