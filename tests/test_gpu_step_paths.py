@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2605_27004_gb300 import inputs
-from gpu_util import gpu_run, oracle_run, perm_lib_to_oracle, rand_theta
+from gpu_util import gpu_run, oracle_run, perm_lib_to_oracle, rand_theta, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -217,6 +217,131 @@ def test_scalar_in_place_makes_no_lists():
     before = torch.cuda.memory_allocated()
     A = lbm.ADE(19, *dims, 0.7, np.eye(3) / 3, solid=solid, storage="fp16s", scheme="aa")
     assert torch.cuda.max_memory_allocated() - before <= A.device_bytes + N + 65536
+
+
+# Every step kernel reports a density that is not positive, in the step that collides it: of the first step
+# (a cell made so) and of the next (a cell of density 100 at a speed of 0.9, whose populations across its
+# motion are negative, -0.2 w of it, and take its neighbours there). One launch is `steps` steps; the cell
+# is the box's last one, so an end of a tile, of a row's second half and of a warp, or one with a fluid
+# neighbour in y and z.
+@pytest.mark.parametrize("q,dims,storage,scheme,frac,steps", [
+    (19, (120, 130, 140), "fp32s", "pull", 0.0, 2), (9, (37, 40, 1), "fp32s", "pull", 0.0, 8),
+    (9, (301, 200, 1), "fp32", "pull", 0.0, 4), (9, (33, 7, 1), "fp64", "pull", 0.0, 1), (9, (33, 7, 1), "fp64", "aa", 0.0, 1),
+    (19, (35, 5, 4), "fp16s", "pull", 0.0, 1), (19, (35, 5, 4), "fp16s", "aa", 0.0, 1), (27, (34, 5, 4), "fp16s", "aa", 0.2, 1),
+    (19, (33, 5, 4), "fp16s", "aa", 0.2, 1), (27, (34, 5, 4), "fp16s", "pull", 0.2, 1), (19, (20, 5, 4), "fp32s", "aa", 0.0, 1)])
+def test_divergence_is_reported(q, dims, storage, scheme, frac, steps):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    d, N = (2 if q == 9 else 3), int(np.prod(dims))
+    solid = inputs.random_mask(N, frac, 4) if frac else np.zeros(N, np.uint8)
+    m = solid.reshape(dims[2], dims[1], dims[0])
+    near = (m == 0) & (np.roll(m, -1, 1) == 0) & (np.roll(m, -1, 0) == 0)  # fluid, as are its neighbours in +y and +z
+    cell = int(np.flatnonzero(near.ravel())[-1])
+    if not frac:
+        assert cell == N - 1
+    L = lbm.LBM(q, *dims, 0.8, np.eye(d) / 3, solid=solid if frac else None, storage=storage, scheme=scheme,
+                check_every=steps, use_graphs=-1)
+
+    def start(rho, u):
+        r, v = torch.ones(N, dtype=L.dtype), torch.zeros(d, N, dtype=L.dtype)
+        r[cell], v[0, cell] = rho, u
+        L.init(r, v)
+
+    def fails():
+        before = L.launches
+        with pytest.raises(lbm.LBMError) as e:
+            L.step(steps)
+        assert e.value.status == -6 and L.launches - before == 1
+
+    start(1.0, 0.05)
+    L.step(2 * steps)
+    start(-1.0, 0.0)
+    fails()
+    start(100.0, 0.9)
+    if steps == 1:
+        L.step(1)
+    fails()
+    if frac:  # what stands in a solid cell is no state
+        r = torch.ones(N, dtype=L.dtype)
+        r[torch.as_tensor(solid != 0)] = float("nan")
+        L.init(r, None)
+        L.step(4)
+
+
+# A flow step, its moments into the scalar's velocity field and the scalar's step, each set up while the one
+# before still runs: against the same calls with a wait after each, bit for bit, and the oracle. The
+# launches queue up behind a bounded spin, so that they do overlap. Boxes of one block an SM at most and
+# of several; a velocity that changes from step to step.
+@pytest.mark.parametrize("storage,scheme", [("fp32s", "pull"), ("fp32s", "aa"), ("fp16s", "pull"), ("fp16s", "aa")])
+@pytest.mark.parametrize("q,dims", [(19, (34, 20, 6)), (9, (30, 40, 1)), (27, (33, 10, 8)), (19, (64, 96, 60)),
+                                    (27, (64, 64, 48)), (9, (200, 1000, 1))])
+def test_coupled_steps_overlap_in_order(q, dims, storage, scheme):
+    import oracle
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    d, N, steps = (2 if q == 9 else 3), int(np.prod(dims)), 11
+    Th, ThS = rand_theta(3, d), rand_theta(4, d)
+    rho0, u0 = inputs.noise_field(N, d, 0.08, 6, rho_amp=0.02)
+    phi0 = 1.0 + 0.5 * np.random.default_rng(2).random(N)
+    F = lbm.LBM(q, *dims, 0.6, Th, storage=storage, scheme=scheme)
+    S = lbm.ADE(q, *dims, 0.7, ThS, storage=storage, scheme=scheme)
+    view = S.velocity_view()
+    got = []
+    for wait in (False, True, False):
+        F.init(torch.as_tensor(rho0), torch.as_tensor(u0))
+        view.zero_()
+        S.init(torch.as_tensor(phi0))
+        torch.cuda.synchronize()
+        if not wait:
+            torch.cuda._sleep(10_000_000)
+        for _ in range(steps):
+            for call in (lambda: F.step(1), lambda: F.moments_into(u=view), lambda: S.step(1)):
+                call()
+                if wait:
+                    torch.cuda.synchronize()
+        got.append((S.scalar(), S.populations(), F.populations()))
+    for g in (got[0], got[2]):
+        assert all(torch.equal(a, b) for a, b in zip(g, got[1]))
+    if N < 10000:
+        Pf = oracle.Problem(q, *dims, 0.6, Th)
+        f = Pf.init(rho0, u0)
+        g = oracle.ADEProblem(q, *dims, 0.7, ThS, np.zeros((d, N))).init_scalar(phi0)
+        for _ in range(steps):
+            Pf.run(f, 1)
+            PS = oracle.ADEProblem(q, *dims, 0.7, ThS, Pf.moments(f)[1])
+            PS.run_scalar(g, 1)
+        tol = 2e-6 if storage == "fp32s" else 1e-3  # as for each of the two alone (40 steps)
+        assert rel_l2(got[0][0].double().cpu().numpy(), PS.scalar(g)) < tol
+
+
+# Held segments with walls (the fluid-cell and sector lists, out of place) and with checkpoints in host
+# memory, copied back ahead of use (room for six states) and not (five).
+@pytest.mark.parametrize("scheme", ["pull", "aa"])
+@pytest.mark.parametrize("frac,states", [(0.2, 0), (0.2, 6), (0.0, 6), (0.0, 5)])
+def test_gradient_with_held_segment_walls_and_host_checkpoints(scheme, frac, states):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    dims, n, K = (18, 7, 6), 20, 5
+    N = int(np.prod(dims))
+    solid = inputs.random_mask(N, frac, 4) if frac else None
+    g = torch.Generator(device="cuda").manual_seed(5)
+    u = 0.03 * torch.randn(3, N, device="cuda", generator=g)
+    w = torch.randn(3, N, device="cuda", generator=g)
+    L = lbm.LBM(19, *dims, 0.7, rand_theta(2, 3), solid=solid, storage="fp16s", scheme=scheme, use_graphs=-1,
+                adjoint_mem_limit=states * 19 * N * 2)
+    L.record_checkpoints(K)
+    runs = []
+    for _ in range(3):
+        L.init(None, u)
+        L.step(n)
+        before = L.launches
+        L.adjoint(w, n, K)
+        runs.append((L.launches - before, L.gradients(), L.populations()))
+        assert (L.adjoint_info()[1] > 0) == (states == 6)
+    for count, (dth, dtau, du0), f in runs[1:]:
+        assert count == runs[0][0] - (K - 1)
+        assert np.array_equal(dth, runs[0][1][0]) and dtau == runs[0][1][1]
+        assert torch.equal(du0, runs[0][1][2]) and torch.equal(f, runs[0][2])
 
 
 def test_slab_group_waits_for_fields_of_the_callers_stream():
