@@ -236,7 +236,9 @@ class SlabGroup:
         failure (the other threads leave at the broken barrier)."""
         import torch
         errs = [None] * self.nslabs
-        for s in self.streams:  # fields made on the caller's stream are read on the slabs' streams
+        # Fields made on the caller's stream are read on the slabs' streams, and memory that the caller's
+        # stream still reads (a gathered part that was freed) is written there.
+        for s in self.streams:
             s.wait_stream(torch.cuda.current_stream(self.device))
 
         def work(r):
@@ -286,8 +288,7 @@ class SlabGroup:
         self._run(lambda r, L: L.step(n))
 
     def record_checkpoints(self, k):
-        for L in self.ctx:
-            L.record_checkpoints(k)
+        self._run(lambda r, L: L.record_checkpoints(k))
 
     def moments(self, Pi=False):
         outs = [None] * self.nslabs
@@ -323,13 +324,16 @@ class SlabGroup:
         self._run(lambda r, L: L.adjoint(g[r], n, checkpoint_every))
 
     def gradients(self):
-        dth, dtau, du0 = 0.0, 0.0, []
-        for L in self.ctx:
-            a, b, c = L.gradients()
+        outs = [None] * self.nslabs
+
+        def g(r, L):
+            outs[r] = L.gradients()
+        self._run(g)
+        dth, dtau = 0.0, 0.0
+        for a, b, _ in outs:
             dth = dth + a
             dtau += b
-            du0.append(c)
-        return dth, dtau, self._gather(du0)
+        return dth, dtau, self._gather([o[2] for o in outs])
 
     @property
     def launches(self):

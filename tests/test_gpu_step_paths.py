@@ -369,6 +369,26 @@ def test_slab_group_waits_for_fields_of_the_callers_stream():
     assert torch.equal(got[0], got[1])
 
 
+def test_slab_group_gradients_wait_for_the_callers_stream():
+    """The slabs' parts of du0 are written on the slabs' streams: not into memory that the caller's stream,
+    held back here by a bounded spin, has yet to write for tensors that are gone."""
+    import torch
+    from paper_2605_27004_gb300 import slabs
+    dims, N = (12, 5, 8), 12 * 5 * 8
+    rho0, u0 = (torch.as_tensor(a, device="cuda") for a in inputs.noise_field(N, 3, 0.05, 3, rho_amp=0.02))
+    G = slabs.SlabGroup(19, *dims, 0.7, rand_theta(1, 3), 2, storage="fp64")
+    G.init(rho0, u0)
+    G.step(4)
+    G.adjoint(u0.clone(), 4, 2)
+    want = G.gradients()[2]
+    for spin in (1, 100_000_000):  # the first pass loads the kernels
+        torch.cuda.synchronize()
+        torch.cuda._sleep(spin)
+        gone = [torch.full((3, G.ctx[0].N), 7.0, dtype=torch.float64, device="cuda") for _ in range(4)]
+        del gone
+        assert torch.equal(G.gradients()[2], want)
+
+
 # From the second gradient on, the forward run leaves its last segment's states in the adjoint's
 # buffers: the same states as recomputed ones, so the same bits as the first gradient. Whole and cut last
 # segments, one of a single step, a run shorter than a segment; both schemes and parities; in between
