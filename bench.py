@@ -262,8 +262,8 @@ def variant(q, n, storage, scheme, kind, steps, warmup, torch, lbm, peak):
 
 def variant_graphs(q, n, storage, scheme, steps, warmup, torch, lbm, peak):
     """lbm_step(K) as a caller issues it, one call for all K steps: boxes up to 2M cells replay
-    CUDA graphs of 16 steps (the library's default), larger ones launch step by step. Device time
-    of the call from CUDA events on the context's stream."""
+    CUDA graphs of 16 steps (the library's default), larger ones launch kernel by kernel (of one step
+    or of two). Device time of the call from CUDA events on the context's stream."""
     L, nf = make_ctx(q, n, storage, scheme, "tg", torch, lbm)
     K = 16 * max(1, steps // 16)
     L.step(16 * max(1, warmup))  # the first call captures the graph

@@ -194,7 +194,7 @@ LBM_OPS_DECL(27, 0) LBM_OPS_DECL(27, 1) LBM_OPS_DECL(27, 2) LBM_OPS_DECL(27, 3) 
 #undef LBM_OPS_DECL
 
 // Deterministic FP64 sum of `nb` partial records of `width` doubles into out[width]
-// (one block, fixed order).
+// (one block per component, fixed order).
 cudaError_t reduce_partials(const double* partials, long long nb, int width, double* out, cudaStream_t s);
 
 }  // namespace lbm

@@ -1,7 +1,8 @@
 // Device code of the anisotropic-equilibrium BGK lattice Boltzmann library (sm_103a).
 //
-// Every kernel runs one thread per lattice cell, x fastest, so that each direction's loads and
-// stores of a warp touch 32 consecutive elements of one structure-of-arrays plane [q][N]
+// The kernels of this file run one thread per lattice cell (those of two, four and a quarter of a cell per
+// thread, and of several steps per launch, stand in the other headers), x fastest, so that each
+// direction's loads and stores of a warp touch 32 consecutive elements of one structure-of-arrays plane [q][N]
 // (coalesced; the x-1/x+1 shifted reads of a warp straddle one extra 32-byte sector that the
 // neighbouring warp reads anyway, and the y/z-shifted rows are re-read from L2). Addresses are a
 // per-direction plane pointer plus a 32-bit in-plane offset built from three wrapped x indices

@@ -29,7 +29,7 @@ struct Launch {
     // while the previous kernel still runs are not spread evenly, so not where an SM gets one to three
     // of them (D3Q19 FP16 64 x 40 x 50, 250 blocks: 3.3 -> 3.6 us a step; D2Q9 301 x 250, 295 blocks: 2.2 ->
     // 2.5; up to four of the D3Q27 FP16 pair blocks: 64 x 40 x 50 4.0 -> 4.2), nor for FP64, bound by the
-    // FP64 pipes of the SMs (D2Q9 128 x 300 8.5 -> 15.4, D3Q27 26 x 23 x 31 15.7 -> 31.7). Larger boxes
+    // FP64 pipes of the SMs (D2Q9 128 x 300 9.8 -> 16.1, D3Q27 26 x 23 x 31 18.2 -> 35.3). Larger boxes
     // gain nothing: beyond 2M cells, FP16 beyond 90 MB of two arrays (D3Q19 130 x 100 x 100 24.3 -> 24.9),
     // D3Q27 beyond 60 (FP32 96 x 70 x 60 11.9 -> 12.1).
     static bool early(const Geom& g, dim3 grid) {
@@ -84,7 +84,8 @@ struct Launch {
     static bool quads(const Geom& g) { return S == 3 && Q != 27 && !g.link && (g.nx % 128) == 0; }
 
     // Rows of odd length, FP16 storage without walls: two cells of a row per thread (lbm_cells2.cuh).
-    // In small 2D boxes half the threads leave SMs without work (301 x 250 2.2 -> 2.4 us a step).
+    // In small 2D boxes half the threads leave SMs without work (301 x 250 2.2 -> 2.4 us a step). For the
+    // scalar there is no such kernel: its rows of odd length run one cell per thread.
     static bool odd_rows(const Geom& g) {
         return S == 3 && !g.link && (g.nx % 2) == 1 && g.nx >= 3 && (Q != 9 || g.N >= 150000u);
     }
@@ -117,7 +118,7 @@ struct Launch {
     }
 
     // D2Q9 FP64: four lanes per cell (lbm_lanes.cuh) while every scheduler (four per SM) gets one warp
-    // at most; with two, 80^2 takes the 4.6 us of one lane per cell, and 96 x 80 5.3.
+    // at most; with two, 80^2 takes the 5.3 us of one lane per cell, and 96 x 80 5.9 instead of 5.3.
     static constexpr bool LANES = S == 1 && Q == 9;
     static bool lanes(const Geom& g) { return !g.link && (g.N + 7) / 8 <= 4u * (uint32_t)sm_count(); }
 

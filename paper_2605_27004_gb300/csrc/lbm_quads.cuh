@@ -171,11 +171,11 @@ __global__ void __launch_bounds__(256, 2)
 // ---------------------------------------------------------------------------------------------
 // AA odd step (state AAODD -> LOCAL), four cells per thread: gather f_i(x) = A[opp i][x - c_i]
 // as in the pull step, scatter f*_i(x) to A[i][x + c_i]. For c_x = +-1 the four targets
-// x0 + c_x .. x0 + 3 + c_x straddle a word boundary: one half, one aligned 4-byte word of two
-// halves, one half (with periodic wrap). Each slot this thread writes holds a population this
-// thread gathered (the one of the opposite direction at the same cell), so the update is in
-// place and race free; elements of the neighbouring words that a thread loads but does not own
-// are never used by it.
+// x0 + c_x .. x0 + 3 + c_x straddle a word boundary: a thread stores its aligned word whole, with one
+// value that the neighbouring lane computed (see below), for the flow and for the scalar. Each slot
+// holds a population that the cell whose value goes there has gathered (the one of the opposite
+// direction), and is written after that, so the update is in place and race free; elements of the
+// neighbouring words that a thread loads but whose cells it does not own are never used by it.
 // ---------------------------------------------------------------------------------------------
 template <int Q, bool ADE = false>
 __global__ void __launch_bounds__(256, 2)

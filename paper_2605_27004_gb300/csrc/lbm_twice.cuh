@@ -222,10 +222,12 @@ inline Tiles twice_tiles(const Geom& g, int slots, long long& walks) {
 // Whether two steps in one launch are faster than two launches. A plane walk of a block takes 3.1 us
 // (9 x 64 cells, two steps) while one step a launch runs at the copy bandwidth, so the split has to
 // fill the SMs: measured ratio of a step's time against the share `full` of the walks that own cells,
-// 512^3 1.28 (0.99), 256^3 1.20 (0.96), 128^3 1.14 (0.86), 176^3 1.11 (0.84), 224^3 1.04 (0.85),
-// 160^3 1.00 (0.77), 144^3 0.94 (0.68). Rows that are not whole sectors make the tiles' edges share
-// sectors (257^3 0.96, 300^3 0.89), and boxes whose two states stay in L2 in good part are faster in
-// single steps (96^3 0.78).
+// 512^3 1.28 (0.99), 256^3 1.20 (0.96), 128^3 1.10 (0.86), 176^3 1.11 (0.84), 224^3 1.04 (0.85),
+// 160^3 1.00 (0.77), 144^3 0.94 (0.68). Rows that are no multiple of 8 cells make the tiles' edges
+// share sectors: 130 x 128^2 0.92, 132^3 0.97, 196^3 0.94, 252^3 0.89, 257^3 0.96, 258 x 256^2 0.86,
+// 260^3 0.95, 300^3 0.89, 380^3 0.92, 508 x 256^2 0.86. Boxes whose two states stay in L2 in good part are
+// faster in single steps where they are cubes (96^3 0.74, 104^3 0.89, 112^3 0.90, 120^3 0.97); some of
+// them would gain (128^2 x 96 1.06, 64 x 144 x 128 1.06), so the line at 1.9M cells is on the safe side.
 inline bool twice_pays(const Geom& g, int slots, Tiles& t) {
     if (g.nx % 8 != 0 || g.N < 1900000u || slots < 1) return false;
     long long walks = 0;
