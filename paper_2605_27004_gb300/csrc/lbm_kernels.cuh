@@ -387,7 +387,12 @@ __device__ __forceinline__ V cdot(Vec3 v, V ax, V ay, V az) {
 // FP16 storage folds 1/tau into the per-cell factors (om drho, om rho, om 4.5 rho), which shortens the
 // dependency chain of every population: its kernels are bound by issued instructions (D3Q27 0.66 ->
 // 0.70 of the copy peak).
-template <int Q, int S, typename V>
+// AFTER sums the momentum defect in a loop of its own behind the relaxation, with the same operations, which
+// leaves the compiler another order: the AA steps without walls gain by it (us a step, D3Q19 64^3 5.95 ->
+// 5.77, 128^3 58.1 -> 55.9, 256^3 420 -> 386, 512^3 3350 -> 3056; D3Q27 256^3 568 -> 542; only 96 x 88 x 80
+// 12.5 -> 12.6), the others lose (pull 64^3 5.45 -> 5.78, 96 x 88 x 80 14.4 -> 15.3; AA with walls 160^3
+// 102 -> 109).
+template <int Q, int S, bool AFTER = false, typename V>
 __device__ __forceinline__ Macro<V> bgk(const Coef<float>& cf, V (&d)[Q]) {
     constexpr bool FOLD = Store<S>::fold_omega;
     Macro<V> m;
@@ -437,7 +442,11 @@ __device__ __forceinline__ Macro<V> bgk(const Coef<float>& cf, V (&d)[Q]) {
         const V plus = mad(rho, J, E), minus = mad(nrho, J, E);
         d[i] = mad(om1, d[i], FOLD ? plus : om * plus);
         d[i + 1] = mad(om1, d[i + 1], FOLD ? minus : om * minus);
-        if (Store<S>::fix_momentum) add_c(v, d[i] - d[i + 1], ex, ey, ez);
+        if (Store<S>::fix_momentum && !AFTER) add_c(v, d[i] - d[i + 1], ex, ey, ez);
+    }
+    if (Store<S>::fix_momentum && AFTER) {
+#pragma unroll
+        for (int k = 0; k < Lat<Q>::P; ++k) add_c(vel<Q>(2 * k + 1), d[2 * k + 1] - d[2 * k + 2], ex, ey, ez);
     }
     if (Store<S>::fix_momentum) {  // removed along 3 w_i c_i
 #pragma unroll
@@ -548,7 +557,7 @@ __device__ __forceinline__ Macro<double> bgk64(const Coef<double>& cf, double (&
 
 // The collision of a flow step on gathered populations: FP64 storage takes them as stored, the others
 // shifted.
-template <int Q, int S>
+template <int Q, int S, bool AFTER = false>
 __device__ __forceinline__ Macro<typename Store<S>::T> collide(const Coef<typename Store<S>::T>& cf,
                                                                typename Store<S>::T (&d)[Q]) {
     if constexpr (S == 1) {
@@ -557,7 +566,7 @@ __device__ __forceinline__ Macro<typename Store<S>::T> collide(const Coef<typena
         F1 e[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) e[i].v = d[i];
-        const Macro<F1> m = bgk<Q, S>(cf, e);
+        const Macro<F1> m = bgk<Q, S, AFTER>(cf, e);
 #pragma unroll
         for (int i = 0; i < Q; ++i) d[i] = e[i].v;
         return {m.drho.v, m.rho.v, m.jx.v, m.jy.v, m.jz.v, m.ux.v, m.uy.v, m.uz.v};
@@ -686,7 +695,7 @@ __global__ void __launch_bounds__(256) k_step_aa(Geom g, Coef<typename Store<S>:
     } else {
         gather<Q, S, MASK, LAYOUT_LOCAL, false, S == 1>(c, lw, cf, src, d);
     }
-    const Macro<T> m = collide<Q, S>(cf, d);
+    const Macro<T> m = collide<Q, S, !MASK>(cf, d);
     if (bad_cell(m)) *flag = 1;
     if (clean)
         aa_store<Q, S, false, ODD, S == 1>(c, 0u, cf, dst, d);
