@@ -314,6 +314,65 @@ def test_coupled_steps_overlap_in_order(q, dims, storage, scheme):
         assert rel_l2(got[0][0].double().cpu().numpy(), PS.scalar(g)) < tol
 
 
+# A flow and a scalar on streams of their own, joined by events, as the caller runs them and as a graph
+# captured over both streams: kernels that may be set up early then have predecessors on two streams.
+@pytest.mark.parametrize("storage,scheme", [("fp32s", "pull"), ("fp16s", "aa")])
+@pytest.mark.parametrize("q,dims", [(19, (34, 20, 6)), (9, (200, 1000, 1))])
+def test_coupled_steps_on_two_streams_and_in_a_graph(q, dims, storage, scheme):
+    import torch
+    from paper_2605_27004_gb300 import lbm
+    d, N, steps = (2 if q == 9 else 3), int(np.prod(dims)), 6
+    rho0, u0 = (torch.as_tensor(a, device="cuda", dtype=torch.float32)
+                for a in inputs.noise_field(N, d, 0.08, 6, rho_amp=0.02))
+    phi0 = 1.0 + 0.5 * torch.as_tensor(np.random.default_rng(2).random(N), device="cuda", dtype=torch.float32)
+    torch.cuda.synchronize()
+    sf, ss = torch.cuda.Stream(), torch.cuda.Stream()
+    F = lbm.LBM(q, *dims, 0.6, rand_theta(3, d), storage=storage, scheme=scheme, stream=sf)
+    S = lbm.ADE(q, *dims, 0.7, rand_theta(4, d), storage=storage, scheme=scheme, stream=ss)
+    view = S.velocity_view()
+
+    def run(wait):
+        F.init(rho0, u0)
+        S.init(phi0)
+        for _ in range(steps):
+            F.step(1)
+            sf.wait_stream(ss)  # the scalar has read the last velocity
+            F.moments_into(u=view)
+            ss.wait_stream(sf)
+            S.step(1)
+            if wait:
+                torch.cuda.synchronize()
+        sf.wait_stream(ss)
+
+    def result():
+        torch.cuda.synchronize()
+        with torch.cuda.stream(ss):
+            g = S.populations()
+        with torch.cuda.stream(sf):
+            f = F.populations()
+        torch.cuda.synchronize()
+        return g, f
+
+    got = []
+    for wait in (True, False):
+        with torch.cuda.stream(ss):
+            view.zero_()
+        torch.cuda.synchronize()
+        run(wait)
+        got.append(result())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=sf):
+        ss.wait_stream(sf)
+        with torch.cuda.stream(ss):
+            view.zero_()
+        run(False)
+    for _ in range(2):
+        graph.replay()
+        got.append(result())
+    for g, f in got[1:]:
+        assert torch.equal(g, got[0][0]) and torch.equal(f, got[0][1])
+
+
 # Held segments with walls (the fluid-cell and sector lists, out of place) and with checkpoints in host
 # memory, copied back ahead of use (room for six states) and not (five).
 @pytest.mark.parametrize("scheme", ["pull", "aa"])
