@@ -184,7 +184,7 @@ struct lbm_ctx {
     // there by the forward run (step_held)
     long long held_t0 = -1;
     int held = 0;
-    long long hold_n = -1;  // the steps of the last adjoint, until a run of as many has held its states
+    long long hold_n = -1;  // the steps of the last adjoint, if it can use held states, until a run has held them
     bool captured = false;  // an lbm_step was captured by the caller: its replays advance the state unseen
     double grad_theta[6] = {0};
     double grad_tau = 0.0;
@@ -1481,7 +1481,7 @@ int lbm_adjoint(lbm_ctx* c, const void* loss_grad, int n, int K) {
     }
     c->grad_tau = c->hout[6];
     c->grads_ready = true;
-    c->hold_n = n;
+    c->hold_n = recorded && flat_plan ? n : -1;  // the plan that can start from held states
     c->last_adj_K2 = longest;
     c->last_adj_prefetch = prefetched;
     release();

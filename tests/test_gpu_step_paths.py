@@ -524,6 +524,10 @@ def test_only_runs_before_a_gradient_are_held():
     L.adjoint(w, n, K)
     again = L.gradients()
     assert torch.equal(again[2], first[2]) and np.array_equal(again[0], first[0]) and again[1] == first[1]
+    # a run shorter than a segment is no recorded segment of its adjoint, which runs it again
+    assert run([9]) == 2
+    L.adjoint(w, 9, K)
+    assert run([9]) == 2
 
 
 # The adjoint's steps add to the gradient records of the step before, and are set up while that one
