@@ -165,9 +165,9 @@ int lbm_record_checkpoints(lbm_ctx* ctx, int checkpoint_every);
  * device. Leaves f(n) in place. Results are read with lbm_gradients. The working set (two lambda
  * arrays, the segment states) is allocated by the first call and kept for later calls (an
  * optimisation loop pays for it once) until lbm_adjoint_release or lbm_destroy. After an adjoint of n
- * steps over recorded checkpoints whose segments fit the device, the next recorded run that reaches n steps leaves the states of its last segment in that
- * working set (unless the caller captures it), and its adjoint does not recompute them.
- * Synchronises. */
+ * steps over recorded checkpoints whose segments fit the device, the next recorded run that reaches n
+ * steps leaves the states of its last segment in that working set (unless the caller captures it),
+ * and its adjoint does not recompute them. Synchronises. */
 int lbm_adjoint(lbm_ctx* ctx, const void* loss_grad, int n, int checkpoint_every);
 
 /* Plan of the last lbm_adjoint: sub_segment = the longest sub-segment of a full segment when
